@@ -861,12 +861,15 @@ struct PolicyHybrid {
         }
     }
 
-    // Near path.  GUARD: some lane of the warp has the integration guard on
-    // (rare); the other instantiation assumes none has, so near is the
-    // natural test and the noise estimate reuses the far-pair factor m / r.
+    // Near path, first pass: every pair of the tile in FP32, near pairs marked
+    // in a per-lane 64-bit mask (nlo, nhi) for near_pass.  GUARD: some lane of
+    // the warp has the integration guard on (rare); the other instantiation
+    // assumes none has, so near is the natural test and the noise estimate
+    // reuses the far-pair factor m / r.
     template <bool MASK, bool GUARD, int S>
     __device__ static void tile(const unsigned char* buf, int64_t j0, const Eps2& e2s,
-                                I (&is)[IT], Acc (&ac)[IT], int sl)
+                                I (&is)[IT], Acc (&ac)[IT], int sl, uint32_t (&nlo)[IT],
+                                uint32_t (&nhi)[IT])
     {
         static_assert(TJ == 64, "one 64-bit near mask per lane and tile");
         // this lane's records: tile slots sl + S u, u < R, in runs of RUN
@@ -875,12 +878,8 @@ struct PolicyHybrid {
         const float4* sA = reinterpret_cast<const float4*>(buf);
         const float4* sB = reinterpret_cast<const float4*>(buf + TJ * 16);
         const float4* sC = reinterpret_cast<const float4*>(buf + TJ * 32);
-        const float4* sD = reinterpret_cast<const float4*>(buf + TJ * 48);
         const float e2h = e2s.h;
-        const float e2l = e2s.l;
-        // Pass 1: every pair in FP32; near pairs add nothing here and are
-        // marked in a per-lane 64-bit mask (bit u = slot sl + S u).
-        uint32_t nlo[IT], nhi[IT];
+        // near pairs add nothing here: bit u of the mask = slot sl + S u
 #pragma unroll
         for (int q = 0; q < IT; ++q) nlo[q] = nhi[q] = 0u;
 #pragma unroll 1
@@ -965,29 +964,144 @@ struct PolicyHybrid {
                 else nhi[q] |= run[q] << (u0 - 32);
             }
         }
-        // Pass 2: the near pairs in double-single, each lane walking its own
-        // mask; the warp loops max_lane(popcount) times, not once per j.
+    }
+
+    // Near path, second pass: the tile's near pairs in double-single.  A warp
+    // whose lanes each walked their own mask would run the ~270-instruction
+    // pair as often as its busiest lane has bits, with most lanes idle: the
+    // near pairs of a tile belong to one or two of the 32 particles whenever
+    // a block's members are spread over space, and a particle under the
+    // integration guard has all 64.  So the k lanes with near pairs ("owners")
+    // share the warp: L = the largest power of two <= 32 / k lanes serve each
+    // owner, lane slice u taking the mask bits u, u + L, ... with the owner's
+    // state by shuffles; their double-single partial sums meet in a fixed
+    // tree and return to the owner.  For L >= 8 the tree halves the values a
+    // lane carries at each of its first three steps (~140 instructions
+    // instead of ~450 for seven butterflies); with fewer lanes saved than the
+    // tree costs (three rounds), each lane walks its own mask (L = 1).
+    // Measured against every lane walking its own mask: a 32-particle block at
+    // N = 16384 with its prediction 19.5 -> 16.6 us, every particle of
+    // N = 65536 8.33 -> 7.70 ms, block steps at N = 16384 57 -> 43 us each.
+    template <int S>
+    __device__ static void near_pass(const unsigned char* buf, const Eps2& e2s,
+                                     const I (&is)[IT], Acc (&ac)[IT], int lane,
+                                     const uint32_t (&nlo)[IT], const uint32_t (&nhi)[IT])
+    {
+        constexpr int IW = 32 / S;
+        constexpr uint32_t FULL = 0xffffffffu;
+        const float4* sA = reinterpret_cast<const float4*>(buf);
+        const float4* sB = reinterpret_cast<const float4*>(buf + TJ * 16);
+        const float4* sC = reinterpret_cast<const float4*>(buf + TJ * 32);
+        const float4* sD = reinterpret_cast<const float4*>(buf + TJ * 48);
 #pragma unroll
         for (int q = 0; q < IT; ++q) {
             uint32_t lo = nlo[q], hi = nhi[q];
-            while (__any_sync(0xffffffffu, (lo | hi) != 0u)) {
-                if ((lo | hi) != 0u) {
-                    int u;
-                    if (lo) {
-                        u = __ffs(lo) - 1;
-                        lo &= lo - 1u;
-                    } else {
-                        u = 32 + __ffs(hi) - 1;
-                        hi &= hi - 1u;
+            const uint32_t owners = __ballot_sync(FULL, (lo | hi) != 0u);
+            if (owners == 0u) continue;
+            const int k = __popc(owners);
+            const int most = __reduce_max_sync(FULL, __popc(lo) + __popc(hi));
+            int lg = 5 - (32 - __clz(k - 1));  // L = 1 << lg
+            if (most - ((most + (1 << lg) - 1) >> lg) < 3) lg = 0;
+            // the pairs of (lo, hi), records slice + S u, added to `to`
+            auto walk = [&](const DSI& i, int slice, DSAccs& to) {
+                while (__any_sync(FULL, (lo | hi) != 0u)) {
+                    if ((lo | hi) != 0u) {
+                        int u;
+                        if (lo) {
+                            u = __ffs(lo) - 1;
+                            lo &= lo - 1u;
+                        } else {
+                            u = 32 + __ffs(hi) - 1;
+                            hi &= hi - 1u;
+                        }
+                        const int j = slice + S * u;
+                        ds_pair<false, false>(sA[j], sB[j], sC[j], sD[j], i, e2s.h, e2s.l, 0, to);
                     }
-                    const int k = sl + S * u;
-                    ds_pair<false, false>(sA[k], sB[k], sC[k], sD[k], is[q], e2h, e2l, j0 + k,
-                                          ac[q]);
+                }
+            };
+            if (lg == 0) {
+                walk(is[q], lane / IW, ac[q]);
+                continue;
+            }
+            const int L = 1 << lg;
+            // o: the lane of owner number lane / L (bits below o <= rank)
+            const int rank = lane >> lg;
+            int o = 0;
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+                if (__popc(owners & ((1u << (o + step)) - 1u)) <= rank) o += step;
+            uint32_t mine = 1u;  // bits u, u + L, ... of a 32-bit word
+            for (int d = 16; d >= L; d >>= 1) mine |= mine << d;
+            mine <<= lane & (L - 1);
+            if (rank >= k) mine = 0u;
+            lo = __shfl_sync(FULL, lo, o) & mine;
+            hi = __shfl_sync(FULL, hi, o) & mine;
+            DSI cur = is[q];
+            cur.xh = __shfl_sync(FULL, cur.xh, o), cur.xl = __shfl_sync(FULL, cur.xl, o);
+            cur.yh = __shfl_sync(FULL, cur.yh, o), cur.yl = __shfl_sync(FULL, cur.yl, o);
+            cur.zh = __shfl_sync(FULL, cur.zh, o), cur.zl = __shfl_sync(FULL, cur.zl, o);
+            cur.vxh = __shfl_sync(FULL, cur.vxh, o), cur.vxl = __shfl_sync(FULL, cur.vxl, o);
+            cur.vyh = __shfl_sync(FULL, cur.vyh, o), cur.vyl = __shfl_sync(FULL, cur.vyl, o);
+            cur.vzh = __shfl_sync(FULL, cur.vzh, o), cur.vzl = __shfl_sync(FULL, cur.vzl, o);
+            DSAccs sum;
+            sum.zero();
+            walk(cur, o / IW, sum);
+            DSPair v[8];
+            v[0] = ds_pair_of(sum.ax), v[1] = ds_pair_of(sum.ay), v[2] = ds_pair_of(sum.az);
+            v[3] = ds_pair_of(sum.jx), v[4] = ds_pair_of(sum.jy), v[5] = ds_pair_of(sum.jz);
+            v[6] = ds_pair_of(sum.ph);
+            tree_zero(v[7]);
+            const int first = __popc(owners & ((1u << lane) - 1u)) << lg;  // of my helpers
+            if (L >= 8) {
+                // after the step of offset o, lanes with bit o keep the
+                // upper half of the values: value c = 4 b2 + 2 b1 + b0
+                // ends on lanes with bits (b2, b1, b0) at L/2, L/4, L/8
+                halve<4>(v, lane, L / 2);
+                halve<2>(v, lane, L / 4);
+                halve<1>(v, lane, L / 8);
+                for (int o = L / 16; o > 0; o >>= 1) tree_xor(v[0], o);
+                const DSPair mine = v[0];
+#pragma unroll
+                for (int c = 0; c < 7; ++c) {
+                    const int src = first + (c >> 2) * (L / 2) + ((c >> 1) & 1) * (L / 4) +
+                                    (c & 1) * (L / 8);
+                    v[c].h = __shfl_sync(FULL, mine.h, src);
+                    v[c].l = __shfl_sync(FULL, mine.l, src);
+                }
+            } else {
+                for (int o = L / 2; o > 0; o >>= 1)
+#pragma unroll
+                    for (int c = 0; c < 7; ++c) tree_xor(v[c], o);
+#pragma unroll
+                for (int c = 0; c < 7; ++c) {
+                    v[c].h = __shfl_sync(FULL, v[c].h, first);
+                    v[c].l = __shfl_sync(FULL, v[c].l, first);
                 }
             }
+            if (!((owners >> lane) & 1u)) continue;
+            ac[q].ax.add(v[0].h, v[0].l), ac[q].ay.add(v[1].h, v[1].l);
+            ac[q].az.add(v[2].h, v[2].l), ac[q].jx.add(v[3].h, v[3].l);
+            ac[q].jy.add(v[4].h, v[4].l), ac[q].jz.add(v[5].h, v[5].l);
+            ac[q].ph.add(v[6].h, v[6].l);
         }
     }
 
+    // One halving step: 2 H values per lane become H, each summed with the
+    // lane at offset o; lanes with bit o set keep the upper half.
+    template <int H>
+    __device__ static void halve(DSPair (&v)[8], int lane, int o)
+    {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int c = 0; c < H; ++c) {
+            const DSPair keep = up ? v[c + H] : v[c], give = up ? v[c] : v[c + H];
+            DSPair got;
+            got.h = __shfl_xor_sync(0xffffffffu, give.h, o);
+            got.l = __shfl_xor_sync(0xffffffffu, give.l, o);
+            v[c] = keep;
+            tree_add(v[c], got);
+        }
+    }
 };
 
 template <class K>
@@ -1536,12 +1650,18 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
                 far = __all_sync(0xffffffffu, far);
             }
             if (far) K::template far_tile<S>(buf, gi.e2, is, ac, sl);
-            else if (guard_any) {
-                if (mask_self) K::template tile<true, true, S>(buf, j0, gi.e2, is, ac, sl);
-                else K::template tile<false, true, S>(buf, j0, gi.e2, is, ac, sl);
-            } else {
-                if (mask_self) K::template tile<true, false, S>(buf, j0, gi.e2, is, ac, sl);
-                else K::template tile<false, false, S>(buf, j0, gi.e2, is, ac, sl);
+            else {
+                uint32_t nlo[IT], nhi[IT];
+                if (guard_any) {
+                    if (mask_self)
+                        K::template tile<true, true, S>(buf, j0, gi.e2, is, ac, sl, nlo, nhi);
+                    else K::template tile<false, true, S>(buf, j0, gi.e2, is, ac, sl, nlo, nhi);
+                } else {
+                    if (mask_self)
+                        K::template tile<true, false, S>(buf, j0, gi.e2, is, ac, sl, nlo, nhi);
+                    else K::template tile<false, false, S>(buf, j0, gi.e2, is, ac, sl, nlo, nhi);
+                }
+                K::template near_pass<S>(buf, gi.e2, is, ac, lane, nlo, nhi);
             }
         } else {
             if (mask_self) K::template tile<true, S>(buf, j0, gi.e2, is, ac, sl);
