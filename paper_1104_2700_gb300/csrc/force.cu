@@ -185,16 +185,17 @@ cudaError_t force_launch(const ForceArgs& a, cudaStream_t s)
     f.st_dt = a.st_dt;
     f.st_hq = a.st_hq;
     f.eta = a.eta;
-    f.jt_lo = a.jt_lo;
-    f.jt_hi = a.jt_hi;
+    f.jt_lo = a.jt_hi > 0 ? a.jt_lo : 0;
+    f.n_tiles = a.jt_hi > 0 ? a.jt_hi - a.jt_lo : a.n_pad / TJ;
+    f.jstride = tile_stride(f.n_tiles);
     f.cta_mode = a.cta_mode && !a.plan.grp_tile0;
     f.n_act_host = a.n_act_host;
     f.idx_map = a.idx_map;
     f.guard_eta = static_cast<float>(HY_GUARD * a.eta);
     f.dyn_chunks = ens ? (a.dyn_chunks < MAX_CHUNKS ? a.dyn_chunks : MAX_CHUNKS) : 0;
     f.queue = a.counters + RLEVELS * a.counter_stride;
-    if (f.jt_hi > 0 && (a.plan.grp_tile0 || f.jt_lo < 0 || f.jt_hi <= f.jt_lo ||
-                        f.jt_hi > f.n_pad / TJ))
+    if (a.jt_hi > 0 && (a.plan.grp_tile0 || a.jt_lo < 0 || a.jt_hi <= a.jt_lo ||
+                        a.jt_hi > f.n_pad / TJ))
         return cudaErrorInvalidValue;
     if (a.prec == Prec::FP64_H6 && !f.snap) return cudaErrorInvalidValue;
     if (is_hybrid(a.prec) &&

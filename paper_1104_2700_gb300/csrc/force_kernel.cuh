@@ -68,9 +68,10 @@ struct ForceParams {
     const double* st_dt;
     double* st_hq;
     double eta;
-    // One system: the j tiles [jt_lo, jt_hi) this launch sums over (its part
-    // of a j-partitioned force); jt_hi = 0 means every tile.
-    int64_t jt_lo, jt_hi;
+    // One system: the n_tiles j tiles from jt_lo on that this launch sums over
+    // (all, or its part of a j-partitioned force), and the walk's stride
+    // (tile_stride, a chain of divisions that no warp need repeat).
+    int64_t jt_lo, n_tiles, jstride;
     // One system: sum small blocks CTA by CTA (see force_kernel)
     int32_t cta_mode;
     // n_act given at launch (>= 0; else read from n_act_dev), and an
@@ -126,6 +127,8 @@ struct PolicyFP64 {
     static constexpr bool GUARDED = false;
     static constexpr int MIN_CTAS = 3;  // registers capped for three CTAs per SM
     static constexpr int CHUNKS = 1;
+    static constexpr int CUT = 8;    // fewest records of a tile a warp may take (0: whole tiles)
+    static constexpr int UNITS = 8;  // parts of tiles per warp that cutting aims at
     static constexpr int NARR = 2;
     __host__ __device__ static constexpr int elem(int a) { return a < 2 ? 32 : 0; }
     static constexpr int TILE_BYTES = TJ * 64;
@@ -155,16 +158,16 @@ struct PolicyFP64 {
         s.vx = v0.x, s.vy = v0.y, s.vz = v1.x;
     }
 
-    // S lanes share each i; lane slice sl takes records sl, sl + S, ...
+    // S lanes share each i; lane slice sl takes records sl + S u, u in [u0, u1)
     template <bool MASK, int S>
     __device__ static void tile(const unsigned char* buf, int64_t j0, const Eps2& e2s,
-                                I (&is)[IT], Acc (&ac)[IT], int sl)
+                                I (&is)[IT], Acc (&ac)[IT], int sl, int u0, int u1)
     {
         const double eps2 = e2s.d;
         const double2* sP = reinterpret_cast<const double2*>(buf);
         const double2* sV = reinterpret_cast<const double2*>(buf + TJ * 32);
 #pragma unroll 2
-        for (int u = 0; u < TJ / S; ++u) {
+        for (int u = u0; u < u1; ++u) {
             const int k = sl + S * u;
             const double2 p0 = sP[2 * k], p1 = sP[2 * k + 1];
             const double2 v0 = sV[2 * k], v1 = sV[2 * k + 1];
@@ -214,6 +217,8 @@ struct PolicyFP64Snap {
     static constexpr bool GUARDED = false;
     static constexpr int MIN_CTAS = 1;
     static constexpr int CHUNKS = 1;
+    static constexpr int CUT = 8;
+    static constexpr int UNITS = 8;
     static constexpr int NARR = 3;
     __host__ __device__ static constexpr int elem(int a) { return a < 3 ? 32 : 0; }
     static constexpr int TILE_BYTES = TJ * 96;
@@ -248,14 +253,14 @@ struct PolicyFP64Snap {
 
     template <bool MASK, int S>
     __device__ static void tile(const unsigned char* buf, int64_t j0, const Eps2& e2s,
-                                I (&is)[IT], Acc (&ac)[IT], int sl)
+                                I (&is)[IT], Acc (&ac)[IT], int sl, int u0, int u1)
     {
         const double eps2 = e2s.d;
         const double2* sP = reinterpret_cast<const double2*>(buf);
         const double2* sV = reinterpret_cast<const double2*>(buf + TJ * 32);
         const double2* sA = reinterpret_cast<const double2*>(buf + TJ * 64);
 #pragma unroll 1
-        for (int u = 0; u < TJ / S; ++u) {
+        for (int u = u0; u < u1; ++u) {
             const int k = sl + S * u;
             const double2 p0 = sP[2 * k], p1 = sP[2 * k + 1];
             const double2 v0 = sV[2 * k], v1 = sV[2 * k + 1];
@@ -320,6 +325,8 @@ struct PolicyMixed {
     static constexpr bool GUARDED = false;
     static constexpr int MIN_CTAS = IT > 1 ? 2 : 3;  // registers capped: 2 or 3 CTAs per SM
     static constexpr int CHUNKS = 1;
+    static constexpr int CUT = 0;  // one FP32 run per tile: a cut would regroup its sums
+    static constexpr int UNITS = 1;
     static constexpr int NARR = 3;
     __host__ __device__ static constexpr int elem(int a) { return a < 2 ? 16 : (a == 2 ? 8 : 0); }
     static constexpr int TILE_BYTES = TJ * 40;
@@ -354,7 +361,7 @@ struct PolicyMixed {
 
     template <bool MASK, int S>
     __device__ static void tile(const unsigned char* buf, int64_t j0, const Eps2& e2s,
-                                I (&is)[IT], Acc (&ac)[IT], int sl)
+                                I (&is)[IT], Acc (&ac)[IT], int sl, int, int)
     {
         const float4* sA = reinterpret_cast<const float4*>(buf);
         const float4* sB = reinterpret_cast<const float4*>(buf + TJ * 16);
@@ -589,8 +596,10 @@ __device__ __forceinline__ void ds_pair(const float4& A, const float4& B, const 
 template <int IT>
 struct PolicyDS {
     static constexpr bool GUARDED = false;
-    static constexpr int MIN_CTAS = 1;
+    static constexpr int MIN_CTAS = 3;  // registers capped for three CTAs per SM
     static constexpr int CHUNKS = 1;
+    static constexpr int CUT = 8;
+    static constexpr int UNITS = 8;
     static constexpr int NARR = 4;
     __host__ __device__ static constexpr int elem(int a) { return a < 4 ? 16 : 0; }
     static constexpr int TILE_BYTES = TJ * 64;
@@ -603,7 +612,7 @@ struct PolicyDS {
 
     template <bool MASK, int S>
     __device__ static void tile(const unsigned char* buf, int64_t j0, const Eps2& e2s,
-                                I (&is)[IT], Acc (&ac)[IT], int sl)
+                                I (&is)[IT], Acc (&ac)[IT], int sl, int u0, int u1)
     {
         const float4* sA = reinterpret_cast<const float4*>(buf);
         const float4* sB = reinterpret_cast<const float4*>(buf + TJ * 16);
@@ -612,7 +621,7 @@ struct PolicyDS {
         const float e2h = e2s.h;
         const float e2l = e2s.l;
 #pragma unroll 1
-        for (int u = 0; u < TJ / S; ++u) {
+        for (int u = u0; u < u1; ++u) {
             const int k = sl + S * u;
             const float4 A = sA[k];
             const float4 B = sB[k];
@@ -706,6 +715,8 @@ struct PolicyHybrid {
     // fit on an SM
     static constexpr int MIN_CTAS = IT > 1 ? 3 : 4;
     static constexpr int CHUNKS = 4;  // tiles of unequal cost
+    static constexpr int CUT = HY_RUN_NEAR;  // near tiles only, at the runs' bounds
+    static constexpr int UNITS = 1;
     static constexpr int NARR = 4;
     __host__ __device__ static constexpr int elem(int a) { return a < 4 ? 16 : 0; }
     static constexpr int TILE_BYTES = TJ * 64;
@@ -868,11 +879,12 @@ struct PolicyHybrid {
     // reuses the far-pair factor m / r.
     template <bool MASK, bool GUARD, int S>
     __device__ static void tile(const unsigned char* buf, int64_t j0, const Eps2& e2s,
-                                I (&is)[IT], Acc (&ac)[IT], int sl, uint32_t (&nlo)[IT],
-                                uint32_t (&nhi)[IT])
+                                I (&is)[IT], Acc (&ac)[IT], int sl, int ulo, int uhi,
+                                uint32_t (&nlo)[IT], uint32_t (&nhi)[IT])
     {
         static_assert(TJ == 64, "one 64-bit near mask per lane and tile");
-        // this lane's records: tile slots sl + S u, u < R, in runs of RUN
+        // this lane's records: tile slots sl + S u, u in [ulo, uhi), in runs of
+        // RUN (ulo and uhi are multiples of it)
         constexpr int R = TJ / S;
         constexpr int RUN = R < HY_RUN_NEAR ? R : HY_RUN_NEAR;
         const float4* sA = reinterpret_cast<const float4*>(buf);
@@ -883,7 +895,7 @@ struct PolicyHybrid {
 #pragma unroll
         for (int q = 0; q < IT; ++q) nlo[q] = nhi[q] = 0u;
 #pragma unroll 1
-        for (int u0 = 0; u0 < R; u0 += RUN) {
+        for (int u0 = ulo; u0 < uhi; u0 += RUN) {
             float ax[IT], ay[IT], az[IT], jx[IT], jy[IT], jz[IT], ph[IT], bs[IT];
             uint32_t run[IT];
 #pragma unroll
@@ -1140,7 +1152,16 @@ __device__ __forceinline__ int64_t owner_warp(int64_t x, int64_t T, int64_t Pu)
 // CTA mode: the most tiles per warp it takes on, and the most entries a
 // thread loads in one batch when CTAs' entries are added (see force_kernel).
 constexpr int64_t CTA_MAX_TILES = 4;
+constexpr int64_t CTA_CUT_MAX = 256;  // CTAs per group up to which tiles are cut
 constexpr int CTA_BATCH = 16;
+
+// Parts the threads of a CTA split a pair of values into (see cta_finish).
+template <class K, int IT, int S>
+__device__ constexpr int cta_parts()
+{
+    constexpr int PAIRS = K::NV * (32 / S) * IT / 2;
+    return PAIRS >= FORCE_WARPS * 32 ? 1 : FORCE_WARPS * 32 / PAIRS;
+}
 
 // Stream-K chunks per warp (largest; policies choose theirs) and the
 // fewest tiles a chunk is cut down to.
@@ -1166,7 +1187,7 @@ struct GroupInfo {
 // all fall to the one or two warps whose stream-K range covers them, and
 // those warps would finish last.  The stride spreads them over the group's
 // whole range, so equal tile counts per warp are also equal work.
-__device__ __forceinline__ int64_t tile_stride(int64_t nt)
+__host__ __device__ __forceinline__ int64_t tile_stride(int64_t nt)
 {
     const uint32_t m = static_cast<uint32_t>(nt);
     if (m <= 8u) return 1;
@@ -1194,15 +1215,15 @@ struct UniformPlan {
     Eps2 e2;
     int GI;
     template <int GI_>
-    __device__ void init(const ForceParams& f)
+    __device__ void init(const ForceParams& f, int na)
     {
         GI = GI_;
-        n_act = f.n_act_host >= 0 ? f.n_act_host : *f.n_act_dev;
-        G = (n_act + GI_ - 1) / GI_;
-        J0 = f.jt_hi > 0 ? f.jt_lo : 0;
-        NT = f.jt_hi > 0 ? f.jt_hi - f.jt_lo : f.n_pad / TJ;
+        n_act = na;
+        G = (na + GI_ - 1) / GI_;
+        J0 = f.jt_lo;
+        NT = f.n_tiles;
         T = G * NT;
-        jstride = tile_stride(NT);
+        jstride = f.jstride;
         e2 = make_eps2(f.eps2);
     }
     __device__ int64_t find(int64_t t, int) const { return t / NT; }
@@ -1231,7 +1252,7 @@ struct ClusterPlan {
     const ForceParams* f;
     int64_t G, T;
     template <int GI_>
-    __device__ void init(const ForceParams& fp)
+    __device__ void init(const ForceParams& fp, int)
     {
         f = &fp;
         G = fp.plan_scalars[0];
@@ -1291,9 +1312,10 @@ __device__ __noinline__ void cta_finish(const ForceParams& f, unsigned char* sme
     using TV = typename K::TV;
     constexpr int VALS = NV * GI;
     constexpr int NTH = FORCE_WARPS * 32;
-    constexpr int PARTS = VALS >= NTH ? 1 : NTH / VALS;
-    static_assert(VALS * sizeof(TV) <= (size_t)K::STAGES * K::TILE_BYTES &&
-                      PARTS * VALS <= (VALS > NTH ? VALS : NTH),
+    constexpr int PAIRS = VALS / 2;  // values are loaded in pairs, 16 bytes
+    constexpr int PARTS = cta_parts<K, IT, S>();
+    static_assert(VALS % 2 == 0 && sizeof(TV) == 8, "two values per 16-byte load");
+    static_assert((VALS + PARTS * VALS) * sizeof(TV) <= (size_t)K::STAGES * K::TILE_BYTES * 2,
                   "a warp's ring holds the CTA-mode sums");
     auto ring_of = [&](int ww) {
         return reinterpret_cast<TV*>(smem + (size_t)ww * WarpSmem<K>::BYTES +
@@ -1319,27 +1341,29 @@ __device__ __noinline__ void cta_finish(const ForceParams& f, unsigned char* sme
     uint32_t* last_flag = reinterpret_cast<uint32_t*>(smem + 64);  // warp 0's barrier block
     const int tid = threadIdx.x;
     const int64_t key = cg * cR;  // slot of the group's first entry
-    // Level 0: this CTA's entry, its warps' sums added in warp order.
-    if (wib == 0) {
-        for (int vi = lane; vi < VALS; vi += 32) {
-            TV x;
-            tree_zero(x);
-#pragma unroll
-            for (int ww = 0; ww < FORCE_WARPS; ++ww) tree_add(x, ring_of(ww)[vi]);
-            tree_store(f.scratch, (size_t)(key + crank) * VALS + vi, x);
-        }
+    TV* part = ring_of(1);
+    TV* fin = ring_of(2);
+    // Level 0: this CTA's entry, its warps' sums added by all threads.
+    for (int vi = tid; vi < VALS; vi += NTH) {
+        static_assert(FORCE_WARPS == 4, "two pairs of warps");
+        TV x = ring_of(0)[vi], y = ring_of(2)[vi];
+        tree_add(x, ring_of(1)[vi]);
+        tree_add(y, ring_of(3)[vi]);
+        tree_add(x, y);
+        if (cR > 1) tree_store(f.scratch, (size_t)(key + crank) * VALS + vi, x);
+        else fin[vi] = x;
     }
     // The entries meet in a tree, as the warps' sums do in warp mode, but
     // each chunk is added by all the threads of its last CTA, each thread
-    // loading at most CTA_BATCH entries of one value in one batch: the
-    // radix is CTA_BATCH times the parts the CTA's threads split a value
-    // into.  Level L entry r sits in slot key + r * RADIX^L, and a chunk's
-    // sum takes its first entry's slot.
+    // loading at most CTA_BATCH entries of one pair of values, all in one
+    // batch (a dependent round trip to another SM's data takes ~1 us, most of
+    // a level): the radix is CTA_BATCH times the parts the CTA's threads
+    // split a pair into.  Level L entry r sits in slot key + r * RADIX^L, and
+    // a chunk's sum takes its first entry's slot.
     constexpr int RADIX = CTA_BATCH * PARTS;
-    TV* part = ring_of(1);
-    TV* fin = ring_of(2);
     int64_t kk = cR, r = crank, stride = 1;
-    for (int level = 0;; ++level) {
+    if (cR == 1) __syncthreads();  // fin is the group's sum
+    for (int level = 0; kk > 1; ++level) {
         // every store of this CTA's entry precedes thread 0's release
         __syncthreads();
         const int64_t chunk = r / RADIX, first = chunk * RADIX;
@@ -1354,26 +1378,35 @@ __device__ __noinline__ void cta_finish(const ForceParams& f, unsigned char* sme
         __syncthreads();
         if (*last_flag == 0u) return;  // the whole CTA: another one carries the chunk on
         // (thread 0's acquire, passed on by the barrier, orders the loads below)
-        const size_t e0 = (size_t)(key + first * stride) * VALS;
-        const size_t es = (size_t)stride * VALS;
-        auto sum_entries = [&](int vi, int u0, int u1) {  // u1 - u0 <= CTA_BATCH
-            TV y[CTA_BATCH];
+        const double2* e0 = reinterpret_cast<const double2*>(
+            f.scratch + (size_t)(key + first * stride) * VALS);
+        const size_t es = (size_t)stride * PAIRS;
+        // entries [u0, u1) of pair vp, u1 - u0 <= CTA_BATCH
+        auto sum_entries = [&](int vp, int u0, int u1, TV* to) {
+            double2 y[CTA_BATCH];
+            const double2* src = e0 + (size_t)u0 * es + vp;
 #pragma unroll
-            for (int k = 0; k < CTA_BATCH; ++k)
-                if (u0 + k < u1) tree_load(f.scratch, e0 + (size_t)(u0 + k) * es + vi, y[k]);
-            TV x;
-            tree_zero(x);
+            for (int k = 0; k < CTA_BATCH; ++k) {
+                y[k] = u0 + k < u1 ? __ldcg(src) : make_double2(0.0, 0.0);
+                src += es;
+            }
+            TV x[2];
+            tree_zero(x[0]), tree_zero(x[1]);
 #pragma unroll
-            for (int k = 0; k < CTA_BATCH; ++k)
-                if (u0 + k < u1) tree_add(x, y[k]);
-            return x;
+            for (int k = 0; k < CTA_BATCH; ++k) {
+                if (u0 + k >= u1) break;
+                tree_add(x[0], tree_bits<TV>(y[k].x));
+                tree_add(x[1], tree_bits<TV>(y[k].y));
+            }
+            to[2 * vp] = x[0];
+            to[2 * vp + 1] = x[1];
         };
         if (PARTS == 1) {
-            for (int vi = tid; vi < VALS; vi += NTH) fin[vi] = sum_entries(vi, 0, cs);
+            for (int vp = tid; vp < PAIRS; vp += NTH) sum_entries(vp, 0, cs, fin);
         } else {
-            if (tid < PARTS * VALS) {
-                const int vi = tid % VALS, pp = tid / VALS;
-                part[pp * VALS + vi] = sum_entries(vi, cs * pp / PARTS, cs * (pp + 1) / PARTS);
+            if (tid < PARTS * PAIRS) {
+                const int vp = tid % PAIRS, pp = tid / PAIRS;
+                sum_entries(vp, cs * pp / PARTS, cs * (pp + 1) / PARTS, part + pp * VALS);
             }
             __syncthreads();
             for (int vi = tid; vi < VALS; vi += NTH) {
@@ -1430,17 +1463,14 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
     constexpr int IW = 32 / S;
     constexpr int GI = IW * IT;
     const int ir = lane % IW, sl = lane / IW;
-    {
-        // Launch variants tuned for different block sizes share one stream:
-        // each works only inside its n_act window (read on the device, so
-        // the host need not know the block size).
-        const int na = f.n_act_host >= 0 ? f.n_act_host : *f.n_act_dev;
-        if (na < f.nact_lo || na >= f.nact_hi) return;
-    }
+    // Launch variants tuned for different block sizes share one stream: each
+    // works only inside its n_act window (read on the device, so the host
+    // need not know the block size).
+    const int na = f.n_act_host >= 0 ? f.n_act_host : *f.n_act_dev;
+    if (na < f.nact_lo || na >= f.nact_hi) return;
     Plan plan;
-    plan.template init<GI>(f);
-    const int64_t T = plan.T;
-    if (T <= 0) return;
+    plan.template init<GI>(f, na);
+    if (plan.T <= 0) return;
     // CTA mode (one system, few groups: at least four CTAs per group).  Group
     // g gets R consecutive CTAs, each a contiguous stretch of its tile walk,
     // cut in four for the CTA's warps.  The warps' sums meet in shared
@@ -1453,14 +1483,39 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
     // (Only the CTA = true build carries it, the small-block launch variant:
     // the code of its reduction, present in the large-block build, cost that
     // build ~2 % through the register allocation of its tile loops.)
+    //
+    // Cut tiles.  A tile may be cut into 2^wl units of equal records, each
+    // staged and summed on its own.  HYBRID, small blocks: while a launch has
+    // more warps than tiles, one tile per warp leaves most of the chip idle
+    // and the launch as long as its dearest tile.  Near tiles are cut then;
+    // the far loop's FP32 run of 64 is not: one unit does the whole tile, the
+    // others nothing (which one rotates with the tile, since unit u of a tile
+    // is warp u of a CTA and a CTA's warps sit on different schedulers).  DS
+    // and FP64, whose tiles are long (64 x ~250 dependent operations, ~15 us
+    // for a warp alone): until each warp has UNITS units, so that the last
+    // round of tiles is not mostly idle.
+    constexpr bool CUTS = K::CUT > 0 && (CTA || K::UNITS > 1) && TJ / S >= 2 * K::CUT;
+    int wl = 0;
+    auto cut = [&](int64_t tiles, int64_t most, int64_t level) {
+        // (from four units on, not past `level`: more entries than one level
+        // of the CTAs' tree adds cost more than the shorter units save)
+        if constexpr (CUTS)
+            while ((TJ / S >> (wl + 1)) >= K::CUT && (tiles << (wl + 1)) <= most &&
+                   (wl < 2 || (tiles << wl) > level || (tiles << (wl + 1)) <= level))
+                ++wl;
+    };
     bool cta = false;
     int64_t cg = 0, cR = 1, crank = 0;
     if constexpr (Plan::CHUNKED && CTA) {
         if (f.cta_mode && 4 * plan.G <= (int64_t)gridDim.x) {
-            const int64_t rmax = (plan.NT + FORCE_WARPS - 1) / FORCE_WARPS;
+            const int64_t per = gridDim.x / static_cast<uint32_t>(plan.G);
+            cut(plan.NT, K::UNITS * FORCE_WARPS * (per < CTA_CUT_MAX ? per : CTA_CUT_MAX),
+                FORCE_WARPS * CTA_BATCH * cta_parts<K, IT, S>());
+            const int64_t rmax = ((plan.NT << wl) + FORCE_WARPS - 1) / FORCE_WARPS;
             cR = gridDim.x / static_cast<uint32_t>(plan.G);  // G < gridDim.x / 4
             if (cR > rmax) cR = rmax;
             cta = plan.NT <= cR * FORCE_WARPS * CTA_MAX_TILES;
+            if (!cta) wl = 0;
         }
         if (cta) {
             cg = blockIdx.x / static_cast<uint32_t>(cR);
@@ -1468,7 +1523,9 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
             if (cg >= plan.G) return;  // the whole CTA: no group left for it
         }
     }
-    // The flattened (group, tile) space is cut into NCH equal chunks (the
+    if (!cta && K::UNITS > 1) cut(plan.T, K::UNITS * P, K::UNITS * P);
+    const int64_t T = plan.T << wl;  // units
+    // The flattened (group, unit) space is cut into NCH equal chunks (the
     // stream-K split) and warp w takes chunks w, w + P, ...: KC chunks from
     // KC stretches of the space, so that regions of dearer tiles (the near
     // tiles of the hybrid precision crowd where the particles do) are shared
@@ -1551,40 +1608,44 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
     if constexpr (Plan::CHUNKED) {
         if (cta) {
             int64_t c0, c1;
-            if (plan.NT * cR < 0x7fffffff) {  // 32-bit divisions: much shorter
-                const uint32_t nt = static_cast<uint32_t>(plan.NT), r = static_cast<uint32_t>(cR);
+            const int64_t nu = plan.NT << wl;
+            if (nu * cR < 0x7fffffff) {  // 32-bit divisions: much shorter
+                const uint32_t nt = static_cast<uint32_t>(nu), r = static_cast<uint32_t>(cR);
                 c0 = nt * static_cast<uint32_t>(crank) / r;
                 c1 = nt * static_cast<uint32_t>(crank + 1) / r;
             } else {
-                c0 = plan.NT * crank / cR;
-                c1 = plan.NT * (crank + 1) / cR;
+                c0 = nu * crank / cR;
+                c1 = nu * (crank + 1) / cR;
             }
             const int64_t len = c1 - c0;
-            t0 = cg * plan.NT + c0 + len * wib / FORCE_WARPS;
-            t1 = cg * plan.NT + c0 + len * (wib + 1) / FORCE_WARPS;
+            t0 = cg * nu + c0 + len * wib / FORCE_WARPS;
+            t1 = cg * nu + c0 + len * (wib + 1) / FORCE_WARPS;
         }
     }
     // Compute cursor (g, gi) and load cursor (lg, lgi): both start at the
     // group of tile t0; the load cursor runs STAGES tiles ahead.
-    int64_t g = cta ? cg : plan.find(t0, lane);
+    // (t counts units: unit t of a group is part t mod 2^wl of tile t >> wl)
+    int64_t g = cta ? cg : plan.find(t0 >> wl, lane);
     GroupInfo gi = plan.group(g);
     int64_t lg = g;
     GroupInfo lgi = gi;
     int64_t tl = t0;
-    int32_t lpos = static_cast<int32_t>(tile_at(lgi, tl - lgi.tile0));  // j tile of the next load
+    int32_t lpos = static_cast<int32_t>(tile_at(lgi, (tl >> wl) - lgi.tile0));  // j tile of the next load
     auto issue_next = [&]() {
-        if (tl >= lgi.tile0 + lgi.ntiles) {
-            while (tl >= lgi.tile0 + lgi.ntiles) lgi = plan.group(++lg);
-            lpos = static_cast<int32_t>(tile_at(lgi, tl - lgi.tile0));
+        if ((tl >> wl) >= lgi.tile0 + lgi.ntiles) {
+            while ((tl >> wl) >= lgi.tile0 + lgi.ntiles) lgi = plan.group(++lg);
+            lpos = static_cast<int32_t>(tile_at(lgi, (tl >> wl) - lgi.tile0));
         }
         const int s = static_cast<int>(issued % K::STAGES);
         // (self-test: with unfed_first_tile the warp's first tile is never
         // staged, so its barrier never completes and the bounded wait runs out)
         if (lane == 0 && !(f.unfed_first_tile && issued == 0))
             issue_tile<K>(f, ring + s * K::TILE_BYTES, &bars[s], lgi.jtile0 + lpos);
-        lpos += lgi.jstride;
-        if (lpos >= lgi.ntiles) lpos -= lgi.ntiles;
         ++tl;
+        if (!CUTS || (tl & ((1 << wl) - 1)) == 0) {
+            lpos += lgi.jstride;
+            if (lpos >= lgi.ntiles) lpos -= lgi.ntiles;
+        }
         ++issued;
     };
     // the ring is empty at a chunk's start: every staged tile was consumed
@@ -1598,13 +1659,13 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
         const uint32_t k = used;
         const int s = static_cast<int>(k % K::STAGES);
         const uint32_t parity = static_cast<uint32_t>((k / K::STAGES) & 1);
-        while (t >= gi.tile0 + gi.ntiles) {
+        while ((t >> wl) >= gi.tile0 + gi.ntiles) {
             gi = plan.group(++g);
             fresh = true;
         }
         if (fresh) {
             fresh = false;
-            cpos = static_cast<int32_t>(tile_at(gi, t - gi.tile0));
+            cpos = static_cast<int32_t>(tile_at(gi, (t >> wl) - gi.tile0));
             load_group(gi);
             if constexpr (K::GUARDED) {
                 bool gq = false;
@@ -1629,10 +1690,16 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
             break;
         }
         ++used;
-        const int64_t jt = t - gi.tile0;  // rank of the tile in the group's walk
         const int64_t j0 = (gi.jtile0 + cpos) * TJ;
-        cpos += gi.jstride;
-        if (cpos >= gi.ntiles) cpos -= gi.ntiles;
+        int u0 = 0, u1 = TJ / S;  // this unit's records
+        if constexpr (CUTS) {
+            u0 = (static_cast<int>(t) & ((1 << wl) - 1)) * (TJ / S >> wl);
+            u1 = u0 + (TJ / S >> wl);
+        }
+        if (!CUTS || ((t + 1) & ((1 << wl) - 1)) == 0) {
+            cpos += gi.jstride;
+            if (cpos >= gi.ntiles) cpos -= gi.ntiles;
+        }
         bool self_here = false;
 #pragma unroll
         for (int q = 0; q < IT; ++q)
@@ -1649,23 +1716,29 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
                 for (int q = 0; q < IT; ++q) far &= K::tile_far(buf, is[q], e2h);
                 far = __all_sync(0xffffffffu, far);
             }
-            if (far) K::template far_tile<S>(buf, gi.e2, is, ac, sl);
-            else {
+            if (far) {
+                if (!CUTS || ((t ^ (t >> wl)) & ((1 << wl) - 1)) == 0)
+                    K::template far_tile<S>(buf, gi.e2, is, ac, sl);
+            } else {
                 uint32_t nlo[IT], nhi[IT];
                 if (guard_any) {
                     if (mask_self)
-                        K::template tile<true, true, S>(buf, j0, gi.e2, is, ac, sl, nlo, nhi);
-                    else K::template tile<false, true, S>(buf, j0, gi.e2, is, ac, sl, nlo, nhi);
+                        K::template tile<true, true, S>(buf, j0, gi.e2, is, ac, sl, u0, u1, nlo,
+                                                          nhi);
+                    else K::template tile<false, true, S>(buf, j0, gi.e2, is, ac, sl, u0, u1, nlo,
+                                                          nhi);
                 } else {
                     if (mask_self)
-                        K::template tile<true, false, S>(buf, j0, gi.e2, is, ac, sl, nlo, nhi);
-                    else K::template tile<false, false, S>(buf, j0, gi.e2, is, ac, sl, nlo, nhi);
+                        K::template tile<true, false, S>(buf, j0, gi.e2, is, ac, sl, u0, u1, nlo,
+                                                          nhi);
+                    else K::template tile<false, false, S>(buf, j0, gi.e2, is, ac, sl, u0, u1, nlo,
+                                                          nhi);
                 }
                 K::template near_pass<S>(buf, gi.e2, is, ac, lane, nlo, nhi);
             }
         } else {
-            if (mask_self) K::template tile<true, S>(buf, j0, gi.e2, is, ac, sl);
-            else K::template tile<false, S>(buf, j0, gi.e2, is, ac, sl);
+            if (mask_self) K::template tile<true, S>(buf, j0, gi.e2, is, ac, sl, u0, u1);
+            else K::template tile<false, S>(buf, j0, gi.e2, is, ac, sl, u0, u1);
         }
         __syncwarp();
         if (t + K::STAGES < t1) {
@@ -1673,15 +1746,15 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
             issue_next();
         }
 
-        if (!cta && (jt == gi.ntiles - 1 || t == t1 - 1)) {
+        if (!cta && (t + 1 == (gi.tile0 + gi.ntiles) << wl || t == t1 - 1)) {
             // This warp's share of group g is complete.  The warps that
             // share the group are summed by a radix-RB tree: within each
             // chunk of RB consecutive contributors the last to arrive adds
             // the chunk in order and carries the sum one level up.  Level-L
             // entry r lives in scratch slot key + r * RB^L (the first slot of
             // the chunk it replaces); each level has its own counters.
-            const int64_t wf = owner_warp(gi.tile0, T, NCH);
-            const int64_t wl = owner_warp(gi.tile0 + gi.ntiles - 1, T, NCH);
+            const int64_t wf = owner_warp(gi.tile0 << wl, T, NCH);
+            const int64_t we = owner_warp(((gi.tile0 + gi.ntiles) << wl) - 1, T, NCH);
             constexpr int NV = K::NV;
             using TV = typename K::TV;
             TV v[IT][NV];
@@ -1695,7 +1768,7 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
 #pragma unroll
                     for (int c = 0; c < NV; ++c) tree_xor(v[q][c], o);
             const int64_t key = wf + g;
-            int64_t kk = wl - wf + 1;  // entries at this level
+            int64_t kk = we - wf + 1;  // entries at this level
             int64_t r = ch - wf;       // my entry at this level
             int64_t stride = 1;
             bool final_here = true;

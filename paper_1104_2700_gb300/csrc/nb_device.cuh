@@ -230,6 +230,18 @@ __device__ __forceinline__ void tree_load(const double* base, size_t k, DSPair& 
     const float2 v = __ldcg(reinterpret_cast<const float2*>(base) + k);
     x.h = v.x, x.l = v.y;
 }
+// the 8 bytes of a stored value, loaded as a double
+template <class TV>
+__device__ __forceinline__ TV tree_bits(double x)
+{
+    if constexpr (sizeof(TV) == sizeof(double) && !__is_class(TV)) {
+        return x;
+    } else {
+        TV p;
+        p.h = __int_as_float(__double2loint(x)), p.l = __int_as_float(__double2hiint(x));
+        return p;
+    }
+}
 // a += the same value of the lane lane ^ o (butterfly step; the sum is the
 // same in both lanes, since the addition of two values is symmetric)
 __device__ __forceinline__ void tree_xor(double& a, int o)

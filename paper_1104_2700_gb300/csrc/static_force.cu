@@ -28,7 +28,7 @@ static __device__ __align__(256) unsigned char nb_static_scratch[NB_STATIC_SCRAT
 
 constexpr int STATIC_CTAS_PER_SM = 4;  // fixes the number of warps, hence the scratch size
 constexpr int MAX_DEVICES = 64;
-constexpr size_t CONTROL_BYTES = 256;  // status word, n_act, layout bounds
+constexpr size_t CONTROL_BYTES = 256;  // status word, layout bounds
 
 struct DeviceSetup {
     bool ready = false;
@@ -120,7 +120,12 @@ nb_status setup_device(int dev, DeviceSetup*& out)
         if (per_sm > STATIC_CTAS_PER_SM) per_sm = STATIC_CTAS_PER_SM;
         // The scratch of the split-group sums grows with the number of
         // persistent warps; shrink the grid until the largest system allowed
-        // fits the array, so the limit on n holds whatever the SM count.
+        // fits the array, so the limit on n holds whatever the SM count: by
+        // whole CTAs per SM first (350 CTAs on 152 SMs, where 304 fit evenly,
+        // cost a block of 500 of 8192 particles 12 us of its 60).
+        while (per_sm > 1 &&
+               plan_for(NB_STATIC_MAX_N, per_sm * sms).total > NB_STATIC_SCRATCH_BYTES)
+            --per_sm;
         int grid = per_sm * sms;
         while (grid > 1 && plan_for(NB_STATIC_MAX_N, grid).total > NB_STATIC_SCRATCH_BYTES)
             grid -= grid / 8 > 0 ? grid / 8 : 1;
@@ -164,7 +169,6 @@ extern "C" nb_status nb_force_static(int64_t n, const double* m, const double* r
     if (n_act == 0) return NB_OK;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     uint32_t* status = reinterpret_cast<uint32_t*>(s->base);
-    int32_t* n_act_dev = reinterpret_cast<int32_t*>(s->base + 4);
     uint32_t* bound = reinterpret_cast<uint32_t*>(s->base + 8);
     uint32_t* counters = reinterpret_cast<uint32_t*>(s->base + p.counters);
     float4* L = reinterpret_cast<float4*>(s->base + p.layout);
@@ -174,7 +178,6 @@ extern "C" nb_status nb_force_static(int64_t n, const double* m, const double* r
     if (cudaMemsetAsync(status, 0, 4 * sizeof(uint32_t), cs) != cudaSuccess) return NB_ECUDA;
     if (cudaMemsetAsync(counters, 0, p.counter_words * sizeof(uint32_t), cs) != cudaSuccess)
         return NB_ECUDA;
-    if (nb::set_scalars_launch(n_act_dev, n_act, nullptr, 0.0, cs) != cudaSuccess) return NB_ECUDA;
     if (nb::bounds_launch(r, v, 3 * n, bound, cs) != cudaSuccess) return NB_ECUDA;
     static_layout_kernel<<<static_cast<unsigned>((p.n_pad + 255) / 256), 256, 0, cs>>>(
         n, p.n_pad, m, r, v, G, bound, L, L + p.n_pad, L + 2 * p.n_pad, L + 3 * p.n_pad);
@@ -186,7 +189,6 @@ extern "C" nb_status nb_force_static(int64_t n, const double* m, const double* r
     f.n = n;
     f.n_pad = p.n_pad;
     f.idx = idx;
-    f.n_act_dev = n_act_dev;
     f.acc = acc;
     f.jerk = jerk;
     f.pot = pot;
@@ -196,6 +198,8 @@ extern "C" nb_status nb_force_static(int64_t n, const double* m, const double* r
     f.status = status;
     f.eps2 = eps * eps;
     f.grid = s->grid;
+    f.n_act_host = n_act;
+    f.cta_mode = 1;
     if (nb::force_launch(f, cs) != cudaSuccess) return NB_ECUDA;
     uint32_t host_status = 0;
     if (cudaMemcpyAsync(&host_status, status, sizeof(host_status), cudaMemcpyDeviceToHost, cs) !=
