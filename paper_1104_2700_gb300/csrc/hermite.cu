@@ -9,20 +9,9 @@
 
 #include "nb_device.cuh"
 #include "nb_launch.h"
+#include "predict.cuh"
 
 namespace nb {
-
-// Order-preserving map of doubles to unsigned 64-bit keys (for atomicMin).
-__device__ __forceinline__ unsigned long long dkey(double x)
-{
-    const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
-    return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
-__device__ __forceinline__ double dkey_decode(unsigned long long k)
-{
-    const unsigned long long b = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
-    return __longlong_as_double(static_cast<long long>(b));
-}
 
 // ---------------------------------------------------------------------------
 // Steps 2-3: Taylor predictor (Eqs. xpred, vpred) for every j particle, in
@@ -109,234 +98,102 @@ __global__ void predict_h6_kernel(const StateDev st, const JLayout jl, const dou
     A[1] = make_double2(ap[2], 0.0);
 }
 
-// ---------------------------------------------------------------------------
-// Steps 2-3 for the precisions whose j layout holds double-single values
-// (MIXED, DS, HYBRID): the prediction in double-single arithmetic on the
-// FP32 pipes.  GB300 spends ~68 cycles on each FP64 warp instruction, and the
-// FP64 Horner form plus the FP64 split into the layout took ~80 of them per
-// particle, so over a large system (an ensemble predicts every particle at
-// each block step) the predictor was FP64-bound.  Here each FP64 state value
-// is cut into hi + lo floats with integer operations on its bits (hi: the
-// leading 24 significand bits; lo: the remaining 29 rounded to a float, so
-// hi + lo keeps ~48 bits), Eqs. xpred and vpred run as double-single Horner
-// steps (FMA-based TwoProd and TwoSum), and the grid-aligned split is taken
-// from the double-single result.  The layout agrees with an FP64 prediction
-// to its own resolution (~2^-47 of the bound); values far outside the
-// layout's range (|x| < 2^-60 or > 2^60, or not finite) take FP64
-// conversions instead.
-// ---------------------------------------------------------------------------
-struct Dsf {
-    float hi, lo;
-};
-
-__device__ __forceinline__ Dsf dsf_of(double x)
-{
-    // work on the two 32-bit words (tests on the whole 64-bit pattern would
-    // become FP64 compares, which cost as much as the conversion they avoid)
-    const unsigned hw = static_cast<unsigned>(__double2hiint(x));
-    const unsigned lw = static_cast<unsigned>(__double2loint(x));
-    const unsigned e = (hw >> 20) & 0x7ffu;
-    if (e - (1023u - 60u) > 120u) {  // zero, |x| < 2^-60 or > 2^60, not finite
-        if (((hw & 0x7fffffffu) | lw) == 0u) return {0.f, 0.f};
-        const float hi = __double2float_rn(x);
-        return {hi, __double2float_rn(x - static_cast<double>(hi))};
-    }
-    const unsigned sign = hw & 0x80000000u;
-    // 52 significand bits: 20 in hw, 32 in lw; hi keeps the leading 23
-    const float hi =
-        __uint_as_float(sign | ((e - 1023u + 127u) << 23) | ((hw & 0xfffffu) << 3) | (lw >> 29));
-    // the remaining 29 significand bits are worth rest * 2^(e - 1075)
-    const unsigned rest = lw & 0x1fffffffu;
-    const float lo = __uint2float_rn(rest) * __uint_as_float((e - 1075u + 127u) << 23);
-    return {hi, sign ? -lo : lo};
-}
-
-__device__ __forceinline__ Dsf dsf_add(Dsf a, Dsf b)
-{
-    float s, e;
-    two_sum(a.hi, b.hi, s, e);
-    e = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
-    const float h = __fadd_rn(s, e);
-    return {h, __fsub_rn(e, __fsub_rn(h, s))};
-}
-
-__device__ __forceinline__ Dsf dsf_fma(Dsf a, Dsf b, Dsf c)  // a b + c
-{
-    float p, e;
-    two_prod(a.hi, b.hi, p, e);
-    e = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e));
-    const float h = __fadd_rn(p, e);
-    return dsf_add({h, __fsub_rn(e, __fsub_rn(h, p))}, c);
-}
-
-__device__ __forceinline__ Dsf dsf_scale(Dsf a, float pow2) { return {a.hi * pow2, a.lo * pow2}; }
-
-// The grid quantum of grid_quantum() as floats, from the bound's bits.
-__device__ __forceinline__ void grid_quantum_f(uint32_t bound_bits, float& q, float& inv_q)
-{
-    const int eb = static_cast<int>((bound_bits >> 23) & 0xff);
-    int e;
-    if (eb == 0 || eb == 255)
-        frexp(2.0 * static_cast<double>(__uint_as_float(bound_bits)), &e);
-    else
-        e = eb - 125;  // 2B = (1.f / 2) 2^(eb - 125), 1.f / 2 in [0.5, 1)
-    q = ldexpf(1.f, e - 23);
-    inv_q = ldexpf(1.f, 23 - e);
-}
-
-// x rounded to a multiple of q (hi) and the rest (lo); x.hi - hi is exact.
-__device__ __forceinline__ void grid_split_ds(Dsf x, float q, float inv_q, float& hi, float& lo)
-{
-    hi = rintf(x.hi * inv_q) * q;
-    lo = __fadd_rn(__fsub_rn(x.hi, hi), x.lo);
-}
-
-// Largest and smallest of a value over the 64 threads of a tile (two
-// warps): butterfly within each warp, then the two warps through shared
-// memory.  Every thread of the block must call it.
-struct TileExtent {
-    float lo[3], hi[3], gm, g23;
-};
-
-__device__ __forceinline__ void tile_extent_reduce(TileExtent& e)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            e.lo[c] = fminf(e.lo[c], __shfl_xor_sync(0xffffffffu, e.lo[c], o));
-            e.hi[c] = fmaxf(e.hi[c], __shfl_xor_sync(0xffffffffu, e.hi[c], o));
-        }
-        e.gm = fmaxf(e.gm, __shfl_xor_sync(0xffffffffu, e.gm, o));
-        e.g23 = fmaxf(e.g23, __shfl_xor_sync(0xffffffffu, e.g23, o));
-    }
-    __shared__ TileExtent other;
-    if (threadIdx.x == 32) other = e;
-    __syncthreads();
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        e.lo[c] = fminf(e.lo[c], other.lo[c]);
-        e.hi[c] = fmaxf(e.hi[c], other.hi[c]);
-    }
-    e.gm = fmaxf(e.gm, other.gm);
-    e.g23 = fmaxf(e.g23, other.g23);
-}
+// One block of four groups of 64 threads per tile of the j layout: group c < 3
+// predicts component c of the tile's particles and group 3 takes their masses
+// and, for HYBRID, (G m)^(2/3).  The records are put together in shared memory
+// and leave in 16-byte stores.  At the sizes where a predictor launch is a
+// large part of a block step it is bound by the fetch of its instructions, each
+// run once by a cold SM (~13 cycles per instruction of straight-line code), so
+// a warp runs one component's ~200 instructions and not three components'
+// ~540 (before: one thread per particle, 5.6 us in a chain of launches at
+// N = 1024).
+constexpr int PRED_THREADS = 4 * TJ;
 
 template <int PREC>
-__global__ void predict_ds_kernel(const StateDev st, const JLayout jl, const double G,
-                                  const unsigned long long* t_bits, const double t_host,
-                                  const int32_t* n_act_dev, const int32_t* jsrc,
-                                  const int32_t* cluster_of)
+__global__ void __launch_bounds__(PRED_THREADS)
+    predict_ds_kernel(const StateDev st, const JLayout jl, const double G,
+                      const unsigned long long* t_bits, const double t_host,
+                      const int32_t* n_act_dev, const int32_t* jsrc, const int32_t* cluster_of)
 {
     constexpr bool HYB = PREC == static_cast<int>(Prec::HYBRID);
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // j-layout slot
-    // (the hybrid layout's tile boxes need every thread of the tile: one
-    // block is one tile, and n_pad is a whole number of tiles)
-    if (q >= st.n_pad) return;
+    constexpr bool MIX = PREC == static_cast<int>(Prec::MIXED);
+    __shared__ __align__(16) float rec[4][TJ * 4];  // the layout's arrays of this tile
+    __shared__ float ext[2][8];                     // HYBRID: the extents of the two half tiles
+    const int c = threadIdx.x / TJ, slot = threadIdx.x % TJ;
+    const int64_t q = (int64_t)blockIdx.x * TJ + slot;  // j-layout slot (n_pad: whole tiles)
     const int64_t n = st.n;
-    const int64_t i = jsrc ? jsrc[q] : (q < n ? q : -1);
-    // an empty block step writes nothing; the ghosts' check is cheap, the
-    // particles' comes after their state loads so that they need not wait
-    if (i < 0 && !HYB) {  // a ghost: far away, zero mass
-        if (n_act_dev && *n_act_dev == 0) return;
-        const float g = static_cast<float>(GHOST_POS);
-        if (PREC == static_cast<int>(Prec::MIXED)) {
-            static_cast<float4*>(jl.arr[0])[q] = make_float4(g, g, g, 0.f);
-            static_cast<float4*>(jl.arr[1])[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            static_cast<float2*>(jl.arr[2])[q] = make_float2(0.f, 0.f);
+    const int64_t i = jsrc ? jsrc[q] : (q < n ? q : -1);  // -1: a ghost
+    float lo_e = CUDART_INF_F, hi_e = -CUDART_INF_F;  // the tile's box (a ghost adds nothing)
+    if (c < 3) {
+        float hi = static_cast<float>(GHOST_POS), lo = 0.f;
+        Dsf v = {0.f, 0.f};
+        if (i >= 0) {
+            const int64_t e = c * n + i;
+            const double x0 = st.x[e], v0 = st.v[e], a0 = st.a[e], j0 = st.j[e], ti = st.t[i];
+            const double t = t_bits ? dkey_decode(t_bits[cluster_of ? cluster_of[i] : 0]) : t_host;
+            float qx, iqx;
+            grid_quantum_f(st.bound[0], qx, iqx);
+            const Dsf h = dsf_of(t - ti);  // exact: both times are dyadic
+            const PredictedComp p = predict_component(x0, v0, a0, j0, h, qx, iqx);
+            hi = p.hi, lo = p.lo, v = p.v;
+            lo_e = hi_e = hi;
+        }
+        rec[0][4 * slot + c] = hi;
+        rec[1][4 * slot + c] = lo;
+        if (MIX) {  // (vx; vy, vz) follow the lo parts
+            const float f = __fadd_rn(v.hi, v.lo);
+            if (c == 0) rec[1][4 * slot + 3] = f;
+            else rec[2][2 * slot + c - 1] = f;
         } else {
-            static_cast<float4*>(jl.arr[0])[q] = make_float4(g, g, g, 0.f);
-            static_cast<float4*>(jl.arr[1])[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            static_cast<float4*>(jl.arr[2])[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            static_cast<float4*>(jl.arr[3])[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            float qv = 0.f, iqv = 0.f, vh, vl;
+            if (!HYB) grid_quantum_f(st.bound[1], qv, iqv);
+            split_velocity<HYB>(v, qv, iqv, vh, vl);
+            rec[2][4 * slot + c] = vh;
+            rec[3][4 * slot + c] = vl;
         }
-        return;
-    }
-    float hi[3], lo[3];
-    Dsf vp[3];
-    Dsf gm = {0.f, 0.f};
-    if (i >= 0) {
-        const double t = t_bits ? dkey_decode(t_bits[cluster_of ? cluster_of[i] : 0]) : t_host;
-        const Dsf h = dsf_of(t - st.t[i]);  // exact: both times are dyadic
-        gm = dsf_fma(dsf_of(G), dsf_of(st.m[i]), Dsf{0.f, 0.f});
-        const Dsf sixth = {0x1.555556p-3f, -0x1.555556p-28f};  // 1/6 to ~2^-50
-        float qx, iqx;
-        grid_quantum_f(st.bound[0], qx, iqx);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const Dsf x = dsf_of(st.x[c * n + i]), v = dsf_of(st.v[c * n + i]);
-            const Dsf a = dsf_of(st.a[c * n + i]), j = dsf_of(st.j[c * n + i]);
-            // Eq. xpred: x + h (v + h (a / 2 + h j / 6)); Eq. vpred: v + h (a + h j / 2)
-            Dsf u = dsf_fma(j, sixth, Dsf{0.f, 0.f});
-            u = dsf_fma(h, u, dsf_scale(a, 0.5f));
-            u = dsf_fma(h, u, v);
-            grid_split_ds(dsf_fma(h, u, x), qx, iqx, hi[c], lo[c]);
-            vp[c] = dsf_fma(h, dsf_fma(h, dsf_scale(j, 0.5f), a), v);
-        }
-    } else {  // a ghost of the hybrid layout
-        hi[0] = hi[1] = hi[2] = static_cast<float>(GHOST_POS);
-        lo[0] = lo[1] = lo[2] = 0.f;
-        vp[0] = vp[1] = vp[2] = Dsf{0.f, 0.f};
-    }
-    if (n_act_dev && *n_act_dev == 0) return;  // the same for every thread
-    if (PREC == static_cast<int>(Prec::MIXED)) {
-        static_cast<float4*>(jl.arr[0])[q] = make_float4(hi[0], hi[1], hi[2], __fadd_rn(gm.hi, gm.lo));
-        static_cast<float4*>(jl.arr[1])[q] =
-            make_float4(lo[0], lo[1], lo[2], __fadd_rn(vp[0].hi, vp[0].lo));
-        static_cast<float2*>(jl.arr[2])[q] =
-            make_float2(__fadd_rn(vp[1].hi, vp[1].lo), __fadd_rn(vp[2].hi, vp[2].lo));
     } else {
-        float vh[3], vl[3];
-        if (HYB) {
-            // the FP32 value of v and the rest: far pairs difference FP32
-            // velocities, near pairs the whole double-single value
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                vh[c] = __fadd_rn(vp[c].hi, vp[c].lo);
-                vl[c] = __fadd_rn(__fsub_rn(vp[c].hi, vh[c]), vp[c].lo);
-            }
+        const Dsf gm = i >= 0 ? dsf_mass(G, st.m[i]) : Dsf{0.f, 0.f};
+        if (MIX) {
+            rec[0][4 * slot + 3] = __fadd_rn(gm.hi, gm.lo);
         } else {
-            float qv, iqv;
-            grid_quantum_f(st.bound[1], qv, iqv);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) grid_split_ds(vp[c], qv, iqv, vh[c], vl[c]);
+            // (G m)^(2/3): the hybrid precision's near-pair test
+            const float g = cbrtf(gm.hi);
+            rec[0][4 * slot + 3] = gm.hi;
+            rec[1][4 * slot + 3] = gm.lo;
+            rec[2][4 * slot + 3] = g * g;
+            rec[3][4 * slot + 3] = 0.f;
+            lo_e = -gm.hi, hi_e = g * g;  // (the largest G m as a smallest -G m)
         }
-        static_cast<float4*>(jl.arr[0])[q] = make_float4(hi[0], hi[1], hi[2], gm.hi);
-        static_cast<float4*>(jl.arr[1])[q] = make_float4(lo[0], lo[1], lo[2], gm.lo);
-        // (G m)^(2/3): the hybrid precision's near-pair test
-        const float g23 = cbrtf(gm.hi);
-        static_cast<float4*>(jl.arr[2])[q] = make_float4(vh[0], vh[1], vh[2], g23 * g23);
-        float box = 0.f;
-        if (HYB) {
-            // the tile's box (hi parts; a ghost adds nothing) and its
-            // largest G m and (G m)^(2/3), for the force kernel's test of
-            // whether a whole tile is far from an i particle.  It rides in
-            // the spare fourth component of the tile's first eight D
-            // records (lo_x, lo_y, lo_z, max G m, hi_x, hi_y, hi_z,
-            // max (G m)^(2/3)), so it arrives with the tile at no extra copy.
-            TileExtent e;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                e.lo[c] = i >= 0 ? hi[c] : CUDART_INF_F;
-                e.hi[c] = i >= 0 ? hi[c] : -CUDART_INF_F;
-            }
-            e.gm = gm.hi;
-            e.g23 = g23 * g23;
-            tile_extent_reduce(e);
-            switch (threadIdx.x) {
-            case 0: box = e.lo[0]; break;
-            case 1: box = e.lo[1]; break;
-            case 2: box = e.lo[2]; break;
-            case 3: box = e.gm; break;
-            case 4: box = e.hi[0]; break;
-            case 5: box = e.hi[1]; break;
-            case 6: box = e.hi[2]; break;
-            case 7: box = e.g23; break;
-            default: break;
-            }
-        }
-        static_cast<float4*>(jl.arr[3])[q] = make_float4(vl[0], vl[1], vl[2], box);
     }
+    if (HYB) {
+        // The tile's box (hi parts) and its largest G m and (G m)^(2/3), for the
+        // force kernel's test of whether a whole tile is far from an i
+        // particle: in the spare fourth component of the tile's first eight D
+        // records (lo_x, lo_y, lo_z, max G m, hi_x, hi_y, hi_z, max
+        // (G m)^(2/3)), so it arrives with the tile at no extra copy.
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) {
+            lo_e = fminf(lo_e, __shfl_xor_sync(0xffffffffu, lo_e, o));
+            hi_e = fmaxf(hi_e, __shfl_xor_sync(0xffffffffu, hi_e, o));
+        }
+        if (slot % 32 == 0) {
+            ext[slot / 32][c] = lo_e;
+            ext[slot / 32][4 + c] = hi_e;
+        }
+    }
+    // an empty block step writes nothing (the same for every thread; checked
+    // after the state loads, so that they need not wait for this one)
+    if (n_act_dev && *n_act_dev == 0) return;
+    __syncthreads();
+    // 16-byte pieces: 64 of each array (MIXED: 64, 64 and 32)
+    float4 w = reinterpret_cast<const float4*>(rec[c])[slot];
+    if (HYB && c == 3 && slot < 8) {
+        const float a = ext[0][slot], b = ext[1][slot];
+        w.w = slot < 3 ? fminf(a, b) : slot == 3 ? -fminf(a, b) : fmaxf(a, b);
+    }
+    const int pieces = MIX ? (c < 2 ? TJ : c == 2 ? TJ / 2 : 0) : TJ;
+    if (slot < pieces)
+        static_cast<float4*>(jl.arr[c])[(int64_t)blockIdx.x * pieces + slot] = w;
 }
 
 // Bounds of the grid-aligned split: max |a_k| and max |b_k| (float bits,
@@ -409,11 +266,11 @@ cudaError_t predict_launch(const StateDev& st, Prec p, const JLayout& jl, double
     case Prec::MIXED:
     case Prec::MIXED_SPJ:  // same j layout
         predict_ds_kernel<static_cast<int>(Prec::MIXED)>
-            <<<blocks, threads, 0, s>>>(st, jl, G, t_bits, t_host, n_act_dev, jsrc, cof);
+            <<<blocks, PRED_THREADS, 0, s>>>(st, jl, G, t_bits, t_host, n_act_dev, jsrc, cof);
         break;
     case Prec::DS:
         predict_ds_kernel<static_cast<int>(Prec::DS)>
-            <<<blocks, threads, 0, s>>>(st, jl, G, t_bits, t_host, n_act_dev, jsrc, cof);
+            <<<blocks, PRED_THREADS, 0, s>>>(st, jl, G, t_bits, t_host, n_act_dev, jsrc, cof);
         break;
     case Prec::FP64_H6:
         if (cl || !st.s || !st.c) return cudaErrorInvalidValue;
@@ -422,7 +279,7 @@ cudaError_t predict_launch(const StateDev& st, Prec p, const JLayout& jl, double
     case Prec::HYBRID:
     case Prec::HYBRID_SPJ:  // same j layout
         predict_ds_kernel<static_cast<int>(Prec::HYBRID)>
-            <<<blocks, threads, 0, s>>>(st, jl, G, t_bits, t_host, n_act_dev, jsrc, cof);
+            <<<blocks, PRED_THREADS, 0, s>>>(st, jl, G, t_bits, t_host, n_act_dev, jsrc, cof);
         break;
     }
     return cudaGetLastError();
