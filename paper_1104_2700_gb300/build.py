@@ -27,8 +27,9 @@ COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-O2",
 PER_FILE = {
     "force.cu": ["-ftz=true"],
     "force_cta.cu": ["-ftz=true"],
+    "force_step.cu": ["-ftz=true"],
 }
-SOURCES = ["capi.cu", "force.cu", "force_cta.cu", "hermite.cu", "static_force.cu", "peak.cu"]
+SOURCES = ["capi.cu", "force.cu", "force_cta.cu", "force_step.cu", "hermite.cu", "static_force.cu", "peak.cu"]
 
 
 def nvcc() -> str:

@@ -670,18 +670,40 @@ nb_status validate_idx(nb_ctx* c, int32_t n_act, const int32_t* idx)
     return NB_OK;
 }
 
+// Whether a block step's select, prediction and force run in one launch: a
+// small system in HYBRID or DS with the default tile shapes.
+bool fused_step(const nb_ctx* c)
+{
+    const nb_ctx::Variant &v0 = c->var[0], &v1 = c->var[1];
+    return !c->ens && c->n <= nb::STEP_MAX_N && nb::force_step_exists(c->prec) && v0.it == 1 &&
+           v0.split == 1 && v1.it == 1 && v1.split == 1 && c->j_parts == 1;
+}
+
 nb_status block_step(nb_ctx* c, double t_end)
 {
     const nb::ClusterDev* cl = c->ens ? &c->cl : nullptr;
     const unsigned long long* tkeys = c->ens ? c->cl.tkey : c->sd.tmin_bits;
-    if (c->ens)
+    const bool fused = fused_step(c);
+    if (fused) {
+        nb::ForceArgs f = force_args(c, c->prec, c->jl, c->sd.idx, c->sd.n_act);
+        f.grid = c->var[0].grid;
+        f.cta_mode = 1;
+        f.fused = true;
+        f.st = c->st;
+        f.sd = c->sd;
+        f.G = c->cfg.G;
+        f.t_end = t_end;
+        NB_CK(c, nb::force_launch(f, c->stream));
+    } else if (c->ens)
         NB_CK(c, nb::cluster_select_launch(c->st, c->cl, c->sd, t_end, c->stream));
     else
         NB_CK(c, nb::select_launch(c->st, c->sd, t_end, c->stream));
-    NB_CK(c, nb::predict_launch(c->st, c->prec, c->jl, c->cfg.G, tkeys, 0.0, c->sd.n_act,
-                                c->stream, cl));
-    nb_status s = run_force_list(c, c->prec, c->jl, c->sd.idx, c->sd.n_act, -1, true);
-    if (s != NB_OK) return s;
+    if (!fused) {
+        NB_CK(c, nb::predict_launch(c->st, c->prec, c->jl, c->cfg.G, tkeys, 0.0, c->sd.n_act,
+                                    c->stream, cl));
+        const nb_status s = run_force_list(c, c->prec, c->jl, c->sd.idx, c->sd.n_act, -1, true);
+        if (s != NB_OK) return s;
+    }
     nb::CorrectArgs ca;
     ca.idx = c->sd.idx;
     ca.n_act_dev = c->sd.n_act;

@@ -125,6 +125,8 @@ int force_ctas_per_sm(Prec p, int it, int split)
     return nb;
 }
 
+bool force_step_exists(Prec p) { return step_kernel_ptr(p) != nullptr; }
+
 size_t force_scratch_doubles(int it, int64_t n_act_max, int warps)
 {
     const int64_t GI = 32 * it;
@@ -147,7 +149,10 @@ int64_t force_counter_entries(int64_t n_act_max, int warps)
 cudaError_t force_launch(const ForceArgs& a, cudaStream_t s)
 {
     const bool ens = a.plan.grp_tile0 != nullptr;
-    const void* fn = kernel_ptr(a.prec, a.it, a.split, ens, a.cta_mode && !ens);
+    const void* fn = a.fused ? step_kernel_ptr(a.prec)
+                             : kernel_ptr(a.prec, a.it, a.split, ens, a.cta_mode && !ens);
+    if (a.fused && (ens || a.it != 1 || a.split != 1 || a.n > STEP_MAX_N || a.jt_hi > 0))
+        return cudaErrorInvalidValue;
     if (!fn || a.grid <= 0) return cudaErrorInvalidValue;
     ForceParams f;
     f.jl0 = a.jl.arr[0];
@@ -201,9 +206,17 @@ cudaError_t force_launch(const ForceArgs& a, cudaStream_t s)
     if (is_hybrid(a.prec) &&
         (!f.st_a || !f.st_j || !f.bound_v || !f.st_dt || !f.st_hq))
         return cudaErrorInvalidValue;
+    if (a.fused) {
+        f.st = a.st;
+        f.G = a.G;
+        f.t_end = a.t_end;
+        f.sel_idx = a.sd.idx;
+        f.sel_n_act = a.sd.n_act;
+        f.sel_tmin = a.sd.tmin_bits;
+    }
     void* args[] = {&f};
     return cudaLaunchKernel(fn, dim3(a.grid), dim3(FORCE_WARPS * 32), args,
-                            force_smem_bytes(a.prec), s);
+                            a.fused ? step_smem_bytes(a.prec) : force_smem_bytes(a.prec), s);
 }
 
 }  // namespace nb

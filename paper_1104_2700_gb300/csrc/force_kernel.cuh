@@ -83,6 +83,13 @@ struct ForceParams {
     // (see force_kernel); the queue word, zero between launches.
     int32_t dyn_chunks;
     uint32_t* queue;
+    // step_force_kernel (force_step.cu) only: the state, G, the end of the
+    // integration, and where the block it selects is published.
+    StateDev st;
+    double G, t_end;
+    int32_t* sel_idx;
+    int32_t* sel_n_act;
+    unsigned long long* sel_tmin;
 };
 
 // A double narrowed to FP32 with integer operations only: the top 23
@@ -607,8 +614,10 @@ struct PolicyDS {
 
     using I = DSI;
     using Acc = DSAccs;
+    static constexpr bool HYB = false;
 
     __device__ static void load_i(const ForceParams& f, int p, int, I& s) { ds_load_i(f, p, s); }
+    __device__ static void limits_i(const ForceParams&, int, I&) {}
 
     template <bool MASK, int S>
     __device__ static void tile(const unsigned char* buf, int64_t j0, const Eps2& e2s,
@@ -725,14 +734,22 @@ struct PolicyHybrid {
 
     using I = HybridI;
     using Acc = HybridAcc;
+    static constexpr bool HYB = true;
 
     __device__ static void load_i(const ForceParams& f, int p, int particle, I& s)
     {
         ds_load_i(f, p, s);
+        limits_i(f, particle, s);
+    }
+
+    // The near radius and the guard of a particle whose position and velocity
+    // are set.
+    __device__ static void limits_i(const ForceParams& f, int particle, I& s)
+    {
         s.ca = s.cj = 0.f;
         s.all_near = false;
         s.particle = particle;
-        if (p < 0) return;
+        if (s.p < 0) return;
         // The near radius and the guard are thresholds, not results: FP32
         // is ample, and the state's doubles are narrowed with integer
         // operations (f32_trunc), so this per-group set-up stays off GB300's
@@ -1297,7 +1314,8 @@ struct ClusterPlan {
 // order as the CTA's entry; the CTAs' entries of group cg added in a tree
 // whose last CTA writes the results.  Kept out of line: inlined, it changed
 // the register allocation of the tile loops and cost ~3 % on large blocks.
-template <class K, int IT, int S>
+// (WSMEM: bytes between the warps' shared-memory areas)
+template <class K, int IT, int S, int WSMEM>
 __device__ __noinline__ void cta_finish(const ForceParams& f, unsigned char* smem,
                                         const typename K::I (&is)[IT],
                                         const typename K::Acc (&ac)[IT], const GroupInfo& cgi,
@@ -1315,11 +1333,10 @@ __device__ __noinline__ void cta_finish(const ForceParams& f, unsigned char* sme
     constexpr int PAIRS = VALS / 2;  // values are loaded in pairs, 16 bytes
     constexpr int PARTS = cta_parts<K, IT, S>();
     static_assert(VALS % 2 == 0 && sizeof(TV) == 8, "two values per 16-byte load");
-    static_assert((VALS + PARTS * VALS) * sizeof(TV) <= (size_t)K::STAGES * K::TILE_BYTES * 2,
+    static_assert(PARTS * VALS * sizeof(TV) <= (size_t)(WSMEM - WarpSmem<K>::BAR_BYTES),
                   "a warp's ring holds the CTA-mode sums");
     auto ring_of = [&](int ww) {
-        return reinterpret_cast<TV*>(smem + (size_t)ww * WarpSmem<K>::BYTES +
-                                     WarpSmem<K>::BAR_BYTES);
+        return reinterpret_cast<TV*>(smem + (size_t)ww * WSMEM + WarpSmem<K>::BAR_BYTES);
     };
     TV v[IT][NV];
 #pragma unroll
@@ -1845,7 +1862,7 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
         if (cta) {
             const GroupInfo cgi = plan.group(cg);
             if (!loaded) load_group(cgi);
-            cta_finish<K, IT, S>(f, smem, is, ac, cgi, cg, cR, crank);
+            cta_finish<K, IT, S, WarpSmem<K>::BYTES>(f, smem, is, ac, cgi, cg, cR, crank);
         }
     }
     (void)aborted;
@@ -1856,5 +1873,10 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
 // lane and a j split of `split`; compiled in their own translation unit
 // (force_cta.cu) so that the two halves of the kernel set build in parallel.
 const void* cta_kernel_ptr(Prec p, int split);
+
+// The kernel of force_step.cu for a precision (null: none) and its CTAs'
+// shared memory.
+const void* step_kernel_ptr(Prec p);
+size_t step_smem_bytes(Prec p);
 
 }  // namespace nb

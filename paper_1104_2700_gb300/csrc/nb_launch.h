@@ -172,6 +172,13 @@ struct ForceArgs {
     // CTA by CTA (shared memory, then one global level) instead of by the
     // warp tree.
     int32_t cta_mode = 0;
+    // One system of at most STEP_MAX_N particles, HYBRID or DS, one i per
+    // lane, no j split: steps 1-4 of a block step to t_end in this launch,
+    // from the state st; the block and its time go to sd.
+    bool fused = false;
+    StateDev st;
+    SchedDev sd;
+    double G = 1.0, t_end = 0.0;
     // n_act known at launch (>= 0): the kernel does not read n_act_dev.
     int32_t n_act_host = -1;
     // Optional: idx holds caller indices, idx_map[i] is the layout slot of i.
@@ -182,6 +189,8 @@ struct ForceArgs {
     int32_t dyn_chunks = 0;
 };
 
+constexpr int STEP_MAX_N = 4096;
+bool force_step_exists(Prec p);
 cudaError_t force_setup(Prec p, int it, int split);  // one-time attribute setup
 int force_ctas_per_sm(Prec p, int it, int split);
 size_t force_smem_bytes(Prec p);
