@@ -4,6 +4,7 @@
 // interpolation, corrector, a0 <- a1, Aarseth timestep in powers of two),
 // the first timesteps and the energy diagnostic.
 #include <cfloat>
+#include <climits>
 #include <math_constants.h>
 #include <cstring>
 
@@ -766,10 +767,12 @@ __device__ __forceinline__ double norm3_rn(double x, double y, double z)
 // taken in FP32: each norm after scaling its vector by a power of two
 // (|v| = nrm 2^E, the vector's largest component then in [0.5, 1)), the two
 // sums after aligning their terms' exponents.  The truncated inputs and about
-// fifteen FP32 roundings leave it within ~2e-6 of the FP64 value, so k is certain unless the value
-// lies within 1e-5 of a power of two; then, or when a vector is zero, tiny or
-// not finite, the function declines and the caller evaluates the formula in
-// FP64 as written.  Either way the timestep chosen is the oracle's.
+// fifteen FP32 roundings leave it within ~2e-6 of the FP64 value, so k is
+// certain unless the value lies within 1e-5 of a power of two; then, or when a
+// vector is zero, tiny or not finite, the function declines and the caller
+// evaluates the formula in FP64 as written.  Either way the timestep chosen is
+// the oracle's.
+
 // A double truncated to a float from its two 32-bit words (within an ulp; a
 // hardware conversion costs as much as an FP64 operation on GB300); values
 // outside [2^-100, 2^100] become 0 or NaN, which the caller's range test
@@ -785,86 +788,93 @@ __device__ __forceinline__ float trunc_to_float(double x)
                            ((hw & 0xfffffu) << 3) | (lw >> 29));
 }
 
-__device__ __forceinline__ bool norm3_scaled(const double (&v)[3], float& nrm, int& E)
+// 2^k as a float for k <= 127; 0 below the normal range.
+__device__ __forceinline__ float pow2f(int k)
 {
-    const float f0 = trunc_to_float(v[0]);
-    const float f1 = trunc_to_float(v[1]);
-    const float f2 = trunc_to_float(v[2]);
-    const float mx = fmaxf(fabsf(f0), fmaxf(fabsf(f1), fabsf(f2)));
-    if (!(mx >= 1e-30f && mx <= 1e30f)) return false;  // NaN fails too
-    frexpf(mx, &E);
-    const float x0 = ldexpf(f0, -E), x1 = ldexpf(f1, -E), x2 = ldexpf(f2, -E);
-    nrm = sqrtf(fmaf(x0, x0, fmaf(x1, x1, x2 * x2)));
-    return true;
+    return k < -126 ? 0.f : __uint_as_float(static_cast<uint32_t>(k + 127) << 23);
 }
 
-__device__ __forceinline__ bool aarseth_interval(const double (&a)[3], const double (&j)[3],
-                                                 const double (&s)[3], const double (&c)[3],
+__device__ __forceinline__ bool norm3_scaled(double v0, double v1, double v2, float& nrm, int& E)
+{
+    const float f0 = trunc_to_float(v0), f1 = trunc_to_float(v1), f2 = trunc_to_float(v2);
+    const float mx = fmaxf(fabsf(f0), fmaxf(fabsf(f1), fabsf(f2)));
+    // (a NaN component must decline; fmaxf would drop it)
+    const bool ok = mx >= 1e-30f && mx <= 1e30f && f0 == f0 && f1 == f1 && f2 == f2;
+    E = static_cast<int>(__float_as_uint(mx) >> 23) - 126;  // mx / 2^E in [0.5, 1)
+    const float sc = pow2f(ok ? -E : 0);
+    const float x0 = f0 * sc, x1 = f1 * sc, x2 = f2 * sc;
+    nrm = sqrtf(fmaf(x0, x0, fmaf(x1, x1, x2 * x2)));
+    return ok;
+}
+
+// The four norms |a|, |j|, |s|, |c| (nrm 2^E) to the interval's exponent.
+__device__ __forceinline__ bool aarseth_interval(const float (&nrm)[4], const int (&E)[4],
                                                  double eta, int& k)
 {
-    float nA, nJ, nS, nC;
-    int eA, eJ, eS, eC;
-    if (!norm3_scaled(a, nA, eA) || !norm3_scaled(j, nJ, eJ) || !norm3_scaled(s, nS, eS) ||
-        !norm3_scaled(c, nC, eC))
-        return false;
+    const float nA = nrm[0], nJ = nrm[1], nS = nrm[2], nC = nrm[3];
     // numerator 2^en (..) and denominator 2^ed (..), each a sum of two
     // positive terms
-    const int n1 = eA + eS, n2 = 2 * eJ, d1 = eJ + eC, d2 = 2 * eS;
+    const int n1 = E[0] + E[2], n2 = 2 * E[1], d1 = E[1] + E[3], d2 = 2 * E[2];
     const int en = n1 > n2 ? n1 : n2, ed = d1 > d2 ? d1 : d2;
-    const float num = ldexpf(nA * nS, n1 - en) + ldexpf(nJ * nJ, n2 - en);
-    const float den = ldexpf(nJ * nC, d1 - ed) + ldexpf(nS * nS, d2 - ed);
+    const float num = nA * nS * pow2f(n1 - en) + nJ * nJ * pow2f(n2 - en);
+    const float den = nJ * nC * pow2f(d1 - ed) + nS * nS * pow2f(d2 - ed);
     int ex = en - ed;
     float r = num / den;
     if (ex & 1) r *= 2.f, ex -= 1;  // an even exponent halves exactly
-    int e;
-    const float m = frexpf(static_cast<float>(eta) * sqrtf(r), &e);  // m in [0.5, 1)
+    const float x = static_cast<float>(eta) * sqrtf(r);
+    const int e = static_cast<int>((__float_as_uint(x) >> 23) & 0xff) - 126;
+    const float m = x * pow2f(-e);  // in [0.5, 1) for a normal x
     if (!(m > 0.500005f && m < 0.99999f)) return false;
     k = e - 1 + ex / 2;
     return k > -1000 && k < 1000;
 }
 
-// Step 8 for one particle: Eq. timestep at the new time (a1, j1, the snap
-// carried to t_next, the crackle), then the power-of-two rule of the
-// hierarchical scheme.  Returns false (and flags the status) when the
-// formula is not a number.
-__device__ __forceinline__ bool next_timestep(const double (&a1)[3], const double (&j1)[3],
-                                              const double (&sn)[3], const double (&c0)[3],
-                                              double h, double tn, const CorrectArgs& c,
-                                              double& dt_new)
+// floor(log2 x) of a positive double (its exponent; -1023 below the normals)
+__device__ __forceinline__ int exponent_of(double x)
 {
-    // cand: min(dt_Aarseth, dt_max), or a power of two in the same
-    // power-of-two interval, which is all the rule below looks at
-    double cand;
-    int kq;
-    const int kmax = static_cast<int>((__double_as_longlong(c.dt_max) >> 52) & 0x7ff) - 1023;
-    if (aarseth_interval(a1, j1, sn, c0, c.eta, kq)) {
-        cand = kq >= kmax ? c.dt_max : __longlong_as_double(static_cast<long long>(kq + 1023) << 52);
+    return static_cast<int>((__double_as_longlong(x) >> 52) & 0x7ff) - 1023;
+}
+
+// Eq. timestep in FP64 as written: min(dt_Aarseth, dt_max), a NaN when the
+// formula is one.  Out of line: it runs only when the FP32 interval declines.
+__device__ __noinline__ double aarseth_fp64(const double (*v)[3][32], int lane, double eta,
+                                            double dt_max)
+{
+    double nrm[4];
+#pragma unroll 1
+    for (int e = 0; e < 4; ++e) nrm[e] = norm3_rn(v[e][0][lane], v[e][1][lane], v[e][2][lane]);
+    // a zero denominator (a particle that feels nothing) sets no constraint
+    const double den = DADD(DMUL(nrm[1], nrm[3]), DMUL(nrm[2], nrm[2]));
+    const double dta =
+        den == 0.0 ? CUDART_INF
+                   : DMUL(eta, __dsqrt_rn(DDIV(DADD(DMUL(nrm[0], nrm[2]), DMUL(nrm[1], nrm[1])), den)));
+    return isnan(dta) ? dta : dta < dt_max ? dta : dt_max;
+}
+
+// The power-of-two rule of the hierarchical scheme (step 8), on exponents: the
+// candidate lies in [2^kq, 2^(kq+1)), the step is h = 2^kh, and the step may
+// double only at a multiple of 2h.  Below the candidate the step is halved
+// until it fits or falls under dt_min.
+__device__ __forceinline__ double pow2_step(int kq, double h, double tn, double dt_min)
+{
+    const int kh = exponent_of(h);
+    const long long b = __double_as_longlong(tn);
+    const int et = static_cast<int>((b >> 52) & 0x7ff);
+    const long long m = (b & 0xfffffffffffffll) | (et ? 1ll << 52 : 0ll);
+    // exponent of the lowest set bit of tn (any power of two divides 0)
+    const int low = m ? (et ? et : 1) - 1075 + __ffsll(m) - 1 : 0x7fffffff;
+    int k;
+    if (kq > kh && low > kh) {
+        k = kh + 1;
+    } else if (kq >= kh) {
+        k = kh;
     } else {
-        const double A = norm3_rn(a1[0], a1[1], a1[2]);
-        const double J = norm3_rn(j1[0], j1[1], j1[2]);
-        const double S = norm3_rn(sn[0], sn[1], sn[2]);
-        const double C = norm3_rn(c0[0], c0[1], c0[2]);
-        // a zero denominator (a particle that feels nothing) sets no constraint
-        const double den = DADD(DMUL(J, C), DMUL(S, S));
-        const double dta =
-            den == 0.0 ? CUDART_INF : DMUL(c.eta, __dsqrt_rn(DDIV(DADD(DMUL(A, S), DMUL(J, J)), den)));
-        if (isnan(dta)) {
-            atomicOr(c.status, ST_NONFINITE);
-            return false;
-        }
-        cand = dta < c.dt_max ? dta : c.dt_max;
+        // smallest power of two >= dt_min
+        const int kmin = exponent_of(dt_min) + ((__double_as_longlong(dt_min) & 0xfffffffffffffll) ? 1 : 0);
+        k = kq > kmin - 1 ? kq : kmin - 1;
+        k = k < kh ? k : kh;
     }
-    dt_new = h;
-    // t_next a multiple of 2h (h a power of two, so t_next / 2h is exact)
-    const double k2h = DMUL(tn, recip_pow2(DMUL(2.0, h)));
-    if (cand >= DMUL(2.0, h) && k2h == rint(k2h)) {
-        dt_new = DMUL(2.0, h);
-    } else if (cand >= h) {
-        dt_new = h;
-    } else {
-        while (dt_new > cand && dt_new >= c.dt_min) dt_new = DMUL(dt_new, 0.5);
-    }
-    return true;
+    return __longlong_as_double(__double_as_longlong(h) + (static_cast<long long>(k - kh) << 52));
 }
 
 __device__ __forceinline__ double pow2_floor(double x)
@@ -876,17 +886,22 @@ __device__ __forceinline__ double pow2_floor(double x)
 
 // GB300's FP64 unit spends ~68 cycles on each warp instruction whatever
 // its number of active lanes, and a warp has one in flight, so a block's
-// latency is the FP64 instruction count of its busiest warp.  A block of
-// three warps therefore takes 32 active particles: warp d does component d
-// of the prediction, snap, crackle and corrector (the bulk of the FP64
-// work), and warp 0 then takes each particle's timestep from the three
-// components left in shared memory.
+// latency is the FP64 instruction count of its busiest warp.  A block of four
+// warps therefore takes 32 active particles: warp d < 3 does component d of
+// the prediction, snap, crackle and corrector (the bulk of the FP64 work); then
+// each of the four warps takes one of the norms of Eq. timestep from shared
+// memory, and warp 0 the steps.  The rest is on exponents and in FP32, and
+// short: a launch runs this code once, and a cold SM fetches straight-line
+// code at ~13 cycles per instruction.
 constexpr int CORR_P = 32;  // particles per block, one per lane
+constexpr int CORR_THREADS = 4 * CORR_P;
 
-__global__ void __launch_bounds__(3 * CORR_P) correct_kernel(const StateDev st, const CorrectArgs c)
+__global__ void __launch_bounds__(CORR_THREADS) correct_kernel(const StateDev st, const CorrectArgs c)
 {
     __shared__ double sv[4][3][CORR_P];  // a1, j1, snap at t_next, crackle
     __shared__ int fin[3][CORR_P];
+    __shared__ float nrm[4][CORR_P];  // scaled norms of the four vectors,
+    __shared__ int nexp[4][CORR_P];   // their exponents (INT_MIN: declined)
     const int d = threadIdx.x / CORR_P, lane = threadIdx.x % CORR_P;
     const int n_act = *c.n_act_dev;
     const int64_t n = st.n;
@@ -921,10 +936,12 @@ __global__ void __launch_bounds__(3 * CORR_P) correct_kernel(const StateDev st, 
             tn = dkey_decode(c.t_bits[c.cluster_of ? c.cluster_of[i] : 0]);
             h = st.dt[i];
             t0 = st.t[i];
-            a1 = c.acc1[3 * k + d];
-            j1 = c.jerk1[3 * k + d];
+            if (d < 3) {
+                a1 = c.acc1[3 * k + d];
+                j1 = c.jerk1[3 * k + d];
+            }
         }
-        fin[d][lane] = isfinite(a1) && isfinite(j1);
+        if (d < 3) fin[d][lane] = isfinite(a1) && isfinite(j1);
         __syncthreads();
         const bool finite = fin[0][lane] && fin[1][lane] && fin[2][lane];
         const bool due = inr && DADD(t0, h) == tn;
@@ -933,7 +950,7 @@ __global__ void __launch_bounds__(3 * CORR_P) correct_kernel(const StateDev st, 
             else if (!finite) atomicOr(c.status, ST_NONFINITE);
         }
         const bool work = due && finite;
-        if (work) {
+        if (work && d < 3) {
             const double dtp = DSUB(tn, t0);
             const double p2 = DMUL(dtp, dtp), p3 = DMUL(p2, dtp);
             const double h2 = DMUL(h, h), h3 = DMUL(h2, h), h4 = DMUL(h3, h), h5 = DMUL(h4, h);
@@ -972,22 +989,38 @@ __global__ void __launch_bounds__(3 * CORR_P) correct_kernel(const StateDev st, 
             sv[3][d][lane] = c0;
         }
         __syncthreads();
+        {
+            float x;
+            int e;
+            if (!norm3_scaled(sv[d][0][lane], sv[d][1][lane], sv[d][2][lane], x, e)) e = INT_MIN;
+            nrm[d][lane] = x;
+            nexp[d][lane] = e;
+        }
+        __syncthreads();
         if (d == 0 && work) {
             st.t[i] = tn;
-            double a3[3], j3[3], s3[3], c3[3];
-#pragma unroll
-            for (int e = 0; e < 3; ++e)
-                a3[e] = sv[0][e][lane], j3[e] = sv[1][e][lane], s3[e] = sv[2][e][lane],
-                c3[e] = sv[3][e][lane];
-            double dt_new;
-            if (next_timestep(a3, j3, s3, c3, h, tn, c, dt_new)) {
+            const float x[4] = {nrm[0][lane], nrm[1][lane], nrm[2][lane], nrm[3][lane]};
+            const int e[4] = {nexp[0][lane], nexp[1][lane], nexp[2][lane], nexp[3][lane]};
+            int kq;
+            bool ok = true;
+            if (e[0] == INT_MIN || e[1] == INT_MIN || e[2] == INT_MIN || e[3] == INT_MIN ||
+                !aarseth_interval(x, e, c.eta, kq)) {
+                const double cand = aarseth_fp64(sv, lane, c.eta, c.dt_max);
+                ok = !isnan(cand);
+                if (!ok) atomicOr(c.status, ST_NONFINITE);
+                kq = exponent_of(cand);
+            }
+            if (ok) {
+                const int kmax = exponent_of(c.dt_max);
+                const double dt_new = pow2_step(kq < kmax ? kq : kmax, h, tn, c.dt_min);
                 st.dt[i] = dt_new;
                 st.nkey[i] = dkey(DADD(tn, dt_new));
                 if (dt_new < c.dt_min) atomicOr(c.status, ST_DTMIN);
             }
         }
-        // fin and sv are written again only after the next iteration's
-        // first barrier has seen warp 0 through its reads
+        // fin and nrm are written again only after the next iteration's
+        // first and second barriers, sv after its first, which have seen warp 0
+        // through its reads
     }
 }
 
@@ -997,7 +1030,7 @@ cudaError_t correct_launch(const StateDev& st, const CorrectArgs& c, cudaStream_
     // enough blocks for every particle to be active; each loops over groups
     const int64_t want = (st.n + CORR_P - 1) / CORR_P;
     const unsigned blocks = static_cast<unsigned>(want < 2432 ? want : 2432);
-    correct_kernel<<<blocks, 3 * CORR_P, 0, s>>>(st, c);
+    correct_kernel<<<blocks, CORR_THREADS, 0, s>>>(st, c);
     return cudaGetLastError();
 }
 
