@@ -403,12 +403,12 @@ nb_status run_force(nb_ctx* c, Prec p, const nb::JLayout& jl, const int32_t* idx
         return NB_OK;
     }
     const nb_ctx::Variant &v0 = c->var[0], &v1 = c->var[1];
-    if (!c->ens && v0.it == 1 && v0.it == v1.it && v0.split == v1.split && v0.grid == v1.grid &&
-        (!nb::is_hybrid(c->prec) || c->n <= ONE_BUILD_MAX_N)) {
+    if (v0.it == v1.it && v0.split == v1.split && v0.grid == v1.grid &&
+        (c->ens || (v0.it == 1 && (!nb::is_hybrid(c->prec) || c->n <= ONE_BUILD_MAX_N)))) {
         f.it = v0.it;
         f.split = v0.split;
         f.grid = v0.grid;
-        f.cta_mode = 1;
+        f.cta_mode = !c->ens;  // (an ensemble's two variants are one build)
         NB_CK(c, nb::force_launch(f, c->stream));
         return NB_OK;
     }

@@ -132,6 +132,7 @@ __device__ __forceinline__ Eps2 make_eps2(double e2)
 template <int IT>
 struct PolicyFP64 {
     static constexpr bool GUARDED = false;
+    static constexpr int PIECE_BYTES = 0;
     static constexpr int MIN_CTAS = 3;  // registers capped for three CTAs per SM
     static constexpr int CHUNKS = 1;
     static constexpr int CUT = 8;    // fewest records of a tile a warp may take (0: whole tiles)
@@ -222,6 +223,7 @@ struct PolicyFP64 {
 template <int IT>
 struct PolicyFP64Snap {
     static constexpr bool GUARDED = false;
+    static constexpr int PIECE_BYTES = 0;
     static constexpr int MIN_CTAS = 1;
     static constexpr int CHUNKS = 1;
     static constexpr int CUT = 8;
@@ -330,6 +332,7 @@ struct PolicyFP64Snap {
 template <int IT, bool SPJ = false>
 struct PolicyMixed {
     static constexpr bool GUARDED = false;
+    static constexpr int PIECE_BYTES = 0;
     static constexpr int MIN_CTAS = IT > 1 ? 2 : 3;  // registers capped: 2 or 3 CTAs per SM
     static constexpr int CHUNKS = 1;
     static constexpr int CUT = 0;  // one FP32 run per tile: a cut would regroup its sums
@@ -603,6 +606,7 @@ __device__ __forceinline__ void ds_pair(const float4& A, const float4& B, const 
 template <int IT>
 struct PolicyDS {
     static constexpr bool GUARDED = false;
+    static constexpr int PIECE_BYTES = 0;
     static constexpr int MIN_CTAS = 3;  // registers capped for three CTAs per SM
     static constexpr int CHUNKS = 1;
     static constexpr int CUT = 8;
@@ -720,6 +724,7 @@ struct HybridAcc : DSAccs {
 template <int IT, bool SPJ = false>
 struct PolicyHybrid {
     static constexpr bool GUARDED = true;
+    static constexpr int PIECE_BYTES = 3584;  // near pairs' partial sums: 63 x 7 x 8 bytes
     // registers capped so that three CTAs (two i per lane) or four (one)
     // fit on an SM
     static constexpr int MIN_CTAS = IT > 1 ? 3 : 4;
@@ -729,7 +734,7 @@ struct PolicyHybrid {
     static constexpr int NARR = 4;
     __host__ __device__ static constexpr int elem(int a) { return a < 4 ? 16 : 0; }
     static constexpr int TILE_BYTES = TJ * 64;
-    static constexpr int STAGES = 3;
+    static constexpr int STAGES = 2;
     static constexpr int NV = 8;  // acc, jerk, pot and the noise estimate
 
     using I = HybridI;
@@ -1006,15 +1011,17 @@ struct PolicyHybrid {
     // state by shuffles; their double-single partial sums meet in a fixed
     // tree and return to the owner.  For L >= 8 the tree halves the values a
     // lane carries at each of its first three steps (~140 instructions
-    // instead of ~450 for seven butterflies); with fewer lanes saved than the
-    // tree costs (three rounds), each lane walks its own mask (L = 1).
+    // instead of ~450 for seven butterflies).  With more than 16 owners, or
+    // fewer rounds saved than the tree costs (three), each lane walks its own
+    // mask, or the warp shares out the list of all pairs (balanced).
     // Measured against every lane walking its own mask: a 32-particle block at
     // N = 16384 with its prediction 19.5 -> 16.6 us, every particle of
     // N = 65536 8.33 -> 7.70 ms, block steps at N = 16384 57 -> 43 us each.
     template <int S>
     __device__ static void near_pass(const unsigned char* buf, const Eps2& e2s,
                                      const I (&is)[IT], Acc (&ac)[IT], int lane,
-                                     const uint32_t (&nlo)[IT], const uint32_t (&nhi)[IT])
+                                     const uint32_t (&nlo)[IT], const uint32_t (&nhi)[IT],
+                                     float2* pieces)
     {
         constexpr int IW = 32 / S;
         constexpr uint32_t FULL = 0xffffffffu;
@@ -1049,7 +1056,20 @@ struct PolicyHybrid {
                 }
             };
             if (lg == 0) {
-                walk(is[q], lane / IW, ac[q]);
+                // many owners: R pairs of the list of all near pairs, owner by
+                // owner, for each lane, if that is shorter than the busiest
+                // lane's own list (instructions: ~290 a pair of one's own,
+                // ~335 one of the list, ~80 a piece brought back)
+                const int mine = __popc(lo) + __popc(hi);
+                const int total = __reduce_add_sync(FULL, mine);
+                const int R = (total + 31) >> 5;
+                const int most_pieces = (most + R - 1) / R + 1;
+                if (R * 335 + most_pieces * 80 + 250 >= most * 290) {
+                    walk(is[q], lane / IW, ac[q]);
+                    continue;
+                }
+                balanced<S>(sA, sB, sC, sD, e2s, is[q], ac[q], lane, lo, hi, owners, mine, total,
+                            R, pieces);
                 continue;
             }
             const int L = 1 << lg;
@@ -1115,6 +1135,112 @@ struct PolicyHybrid {
         }
     }
 
+    // The near pairs of all owners laid end to end, lane l takes [l R, l R + R):
+    // it walks them with the owner's state by shuffles and leaves a sum, a
+    // "piece", at each change of owner.  Piece slots: lane + owner, which grows
+    // strictly along the list, so an owner's pieces are consecutive and meet in
+    // list order.
+    template <int S>
+    __device__ static void balanced(const float4* sA, const float4* sB, const float4* sC,
+                                    const float4* sD, const Eps2& e2s, const I& own, Acc& acc,
+                                    int lane, uint32_t lo, uint32_t hi, uint32_t owners, int mine,
+                                    int total, int R, float2* pieces)
+    {
+        constexpr int IW = 32 / S;
+        constexpr uint32_t FULL = 0xffffffffu;
+        int start = mine;  // exclusive prefix of the counts
+#pragma unroll 1
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(FULL, start, d);
+            if (lane >= d) start += y;
+        }
+        start -= mine;
+        // my first pair's owner: the last lane whose pairs start at or before it
+        const int p0 = lane * R;
+        int o = 0;
+#pragma unroll 1
+        for (int step = 16; step > 0; step >>= 1)
+            if (__shfl_sync(FULL, start, o + step) <= p0) o += step;
+        int left = total - p0;  // pairs left to me
+        left = left < 0 ? 0 : left < R ? left : R;
+        uint32_t clo = __shfl_sync(FULL, lo, o), chi = __shfl_sync(FULL, hi, o);
+        {  // without the owner's pairs before mine
+            int skip = p0 - __shfl_sync(FULL, start, o);
+            const int nl = __popc(clo);
+            if (skip >= nl) {
+                skip -= nl;
+                clo = 0u;
+                chi = drop_bits(chi, skip);
+            } else {
+                clo = drop_bits(clo, skip);
+            }
+        }
+        DSI cur = own;
+        DSAccs sum;
+        sum.zero();
+        auto leave = [&]() {
+            float2* w = pieces + (lane + o) * 7;
+            w[0] = make_float2(sum.ax.hi, sum.ax.lo), w[1] = make_float2(sum.ay.hi, sum.ay.lo);
+            w[2] = make_float2(sum.az.hi, sum.az.lo), w[3] = make_float2(sum.jx.hi, sum.jx.lo);
+            w[4] = make_float2(sum.jy.hi, sum.jy.lo), w[5] = make_float2(sum.jz.hi, sum.jz.lo);
+            w[6] = make_float2(sum.ph.hi, sum.ph.lo);
+        };
+#pragma unroll 1
+        for (int r = 0; r < R; ++r) {
+            const bool next = left > 0 && (clo | chi) == 0u;  // on to the next owner
+            if (next) {
+                leave();
+                sum.zero();
+                o = __ffs(owners & ~((2u << o) - 1u)) - 1;
+            }
+            const uint32_t flo = __shfl_sync(FULL, lo, o), fhi = __shfl_sync(FULL, hi, o);
+            if (next) clo = flo, chi = fhi;
+            cur.xh = __shfl_sync(FULL, own.xh, o), cur.xl = __shfl_sync(FULL, own.xl, o);
+            cur.yh = __shfl_sync(FULL, own.yh, o), cur.yl = __shfl_sync(FULL, own.yl, o);
+            cur.zh = __shfl_sync(FULL, own.zh, o), cur.zl = __shfl_sync(FULL, own.zl, o);
+            cur.vxh = __shfl_sync(FULL, own.vxh, o), cur.vxl = __shfl_sync(FULL, own.vxl, o);
+            cur.vyh = __shfl_sync(FULL, own.vyh, o), cur.vyl = __shfl_sync(FULL, own.vyl, o);
+            cur.vzh = __shfl_sync(FULL, own.vzh, o), cur.vzl = __shfl_sync(FULL, own.vzl, o);
+            if (left > 0) {
+                --left;
+                int u;
+                if (clo) {
+                    u = __ffs(clo) - 1;
+                    clo &= clo - 1u;
+                } else {
+                    u = 32 + __ffs(chi) - 1;
+                    chi &= chi - 1u;
+                }
+                const int j = o / IW + S * u;
+                ds_pair<false, false>(sA[j], sB[j], sC[j], sD[j], cur, e2s.h, e2s.l, 0, sum);
+            }
+        }
+        if (p0 < total) leave();
+        __syncwarp();
+        if (mine > 0) {
+            const int l1 = (start + mine - 1) / R;
+#pragma unroll 1
+            for (int l = start / R; l <= l1; ++l) {
+                const float2* w = pieces + (l + lane) * 7;
+                acc.ax.add(w[0].x, w[0].y), acc.ay.add(w[1].x, w[1].y);
+                acc.az.add(w[2].x, w[2].y), acc.jx.add(w[3].x, w[3].y);
+                acc.jy.add(w[4].x, w[4].y), acc.jz.add(w[5].x, w[5].y);
+                acc.ph.add(w[6].x, w[6].y);
+            }
+        }
+        __syncwarp();
+    }
+
+    // x without its k lowest set bits
+    __device__ static uint32_t drop_bits(uint32_t x, int k)
+    {
+        int at = 0;  // the lowest position with k set bits below it
+#pragma unroll 1
+        for (int step = 16; step > 0; step >>= 1)
+            if (__popc(x & ((1u << (at + step)) - 1u)) <= k) at += step;
+        return k > 0 ? x & ~((1u << at) - 1u) : x;
+    }
+
     // One halving step: 2 H values per lane become H, each summed with the
     // lane at offset o; lanes with bit o set keep the upper half.
     template <int H>
@@ -1136,7 +1262,7 @@ struct PolicyHybrid {
 template <class K>
 struct WarpSmem {
     static constexpr int BAR_BYTES = 128;  // STAGES mbarriers, padded
-    static constexpr int BYTES = BAR_BYTES + K::STAGES * K::TILE_BYTES;
+    static constexpr int BYTES = BAR_BYTES + K::STAGES * K::TILE_BYTES + K::PIECE_BYTES;
 };
 
 template <class K>
@@ -1751,7 +1877,8 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
                     else K::template tile<false, false, S>(buf, j0, gi.e2, is, ac, sl, u0, u1, nlo,
                                                           nhi);
                 }
-                K::template near_pass<S>(buf, gi.e2, is, ac, lane, nlo, nhi);
+                K::template near_pass<S>(buf, gi.e2, is, ac, lane, nlo, nhi,
+                                         reinterpret_cast<float2*>(ring + K::STAGES * K::TILE_BYTES));
             }
         } else {
             if (mask_self) K::template tile<true, S>(buf, j0, gi.e2, is, ac, sl, u0, u1);

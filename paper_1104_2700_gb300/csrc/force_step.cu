@@ -30,7 +30,10 @@ static_assert(STEP_MAX_N <= 32 * ST_THREADS, "a mask bit per key of a thread");
 // tile for the i particles (its first 32 records), the block.
 template <class K>
 struct StepSmem {
-    static constexpr int WARP = WarpSmem<K>::BAR_BYTES + (K::NV * 32 * 8 + 127) / 128 * 128;
+    // (near pairs' pieces and, after the tiles, the sums share an area)
+    static constexpr int SUMS = (K::NV * 32 * 8 + 127) / 128 * 128;
+    static constexpr int WARP =
+        WarpSmem<K>::BAR_BYTES + (SUMS > K::PIECE_BYTES ? SUMS : K::PIECE_BYTES);
     static constexpr int TILE = TJ * 64;
     static constexpr int TILES = ST_WARPS * WARP;
     static constexpr int LIST = TILES + (ST_TILES + 1) * TILE;
@@ -297,7 +300,9 @@ __global__ void __launch_bounds__(ST_THREADS, K::MIN_CTAS) step_force_kernel(con
                             K::template tile<false, false, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1,
                                                               nlo, nhi);
                     }
-                    K::template near_pass<1>(buf, gi.e2, is, ac, lane, nlo, nhi);
+                    K::template near_pass<1>(buf, gi.e2, is, ac, lane, nlo, nhi,
+                                             reinterpret_cast<float2*>(smem + wib * M::WARP +
+                                                                       WarpSmem<K>::BAR_BYTES));
                 } else {
                     if (mask_self) K::template tile<true, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1);
                     else K::template tile<false, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1);
