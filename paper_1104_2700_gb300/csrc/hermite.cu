@@ -433,58 +433,50 @@ __global__ void __launch_bounds__(SCHED_THREADS)
 constexpr int SEL1_THREADS = 1024;
 constexpr int64_t SEL1_MAX_N = 32 * SEL1_THREADS;
 
+// Smallest 64-bit key over the warp.
+__device__ __forceinline__ unsigned long long warp_min_key(unsigned long long k)
+{
+    const uint32_t hi = static_cast<uint32_t>(k >> 32);
+    const uint32_t mh = __reduce_min_sync(0xffffffffu, hi);
+    const uint32_t ml =
+        __reduce_min_sync(0xffffffffu, hi == mh ? static_cast<uint32_t>(k) : 0xffffffffu);
+    return static_cast<unsigned long long>(mh) << 32 | ml;
+}
+
+// BATCH: keys loaded in one round trip (small systems take the short loop: a
+// cold SM pays for every instruction of it).
+template <int BATCH>
 __global__ void __launch_bounds__(SEL1_THREADS)
     select_one_cta_kernel(const unsigned long long* __restrict__ nkey, int64_t n, double t_end,
                           SchedDev sd)
 {
     __shared__ unsigned long long wmin[SEL1_THREADS / 32];
-    __shared__ unsigned long long tkey;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     unsigned long long best = ~0ull;
     uint32_t mask = 0u;
     const int tiles = static_cast<int>((n + SEL1_THREADS - 1) / SEL1_THREADS);  // <= 32
-    // keys in batches of 16 independent loads (one memory round trip each);
+    // keys in batches of independent loads (one memory round trip each);
     // slots past n read as the largest key and never join the mask
-    for (int u0 = 0; u0 < tiles; u0 += 16) {
-        unsigned long long kk[16];
+#pragma unroll 1
+    for (int u0 = 0; u0 < tiles; u0 += BATCH) {
+        unsigned long long kk[BATCH];
 #pragma unroll
-        for (int v = 0; v < 16; ++v) {
-            const int64_t i = tid + static_cast<int64_t>(SEL1_THREADS) * (u0 + v);
-            kk[v] = (u0 + v < tiles && i < n) ? __ldcg(nkey + i) : ~0ull;
+        for (int v = 0; v < BATCH; ++v) {
+            const int i = tid + SEL1_THREADS * (u0 + v);
+            kk[v] = i < n ? __ldcg(nkey + i) : ~0ull;
         }
 #pragma unroll
-        for (int v = 0; v < 16; ++v) {
-            const unsigned long long k = kk[v];
-            if (k < best) {
-                best = k;
-                mask = 1u << (u0 + v);
-            } else if (k == best && k != ~0ull) {
-                mask |= 1u << (u0 + v);
-            }
+        for (int v = 0; v < BATCH; ++v) {
+            if (kk[v] < best) best = kk[v], mask = 0u;
+            if (kk[v] == best) mask |= 1u << (u0 + v);
         }
     }
-    unsigned long long bmin = best;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, bmin, o);
-        bmin = other < bmin ? other : bmin;
-    }
+    unsigned long long bmin = warp_min_key(best);
     if (lane == 0) wmin[wid] = bmin;
     __syncthreads();
-    if (wid == 0) {
-        bmin = wmin[lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, bmin, o);
-            bmin = other < bmin ? other : bmin;
-        }
-        if (lane == 0) {
-            tkey = bmin;
-            *sd.tmin_bits = bmin;
-        }
-    }
-    __syncthreads();
-    if (best != tkey || !(dkey_decode(tkey) <= t_end)) mask = 0u;
+    bmin = warp_min_key(wmin[lane]);
+    if (tid == 0) *sd.tmin_bits = bmin;
+    if (best != bmin || bmin == ~0ull || !(dkey_decode(bmin) <= t_end)) mask = 0u;
     // Ordered compaction: slot of (tile u, warp w, lane) = members before
     // tile u + members of tile u in warps before w + lanes before it.  One
     // ballot per tile (lane u of each warp keeps its warp's ballot of tile
@@ -492,15 +484,16 @@ __global__ void __launch_bounds__(SEL1_THREADS)
     __shared__ int cnt[32 * (SEL1_THREADS / 32)];
     __shared__ int wtot[SEL1_THREADS / 32];
     uint32_t bal = 0u;
+#pragma unroll 1
     for (int u = 0; u < tiles; ++u) {
         const uint32_t b = __ballot_sync(0xffffffffu, (mask >> u) & 1u);
         if (lane == u) bal = b;
-        if (lane == 0) cnt[u * 32 + wid] = __popc(b);
     }
+    if (lane < tiles) cnt[lane * 32 + wid] = __popc(bal);
     __syncthreads();
     const int mine = tid < tiles * 32 ? cnt[tid] : 0;  // entry tid = (u = wid, w = lane)
     int x = mine;
-#pragma unroll
+#pragma unroll 1
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
@@ -510,7 +503,7 @@ __global__ void __launch_bounds__(SEL1_THREADS)
     if (wid == 0) {
         const int c = wtot[lane];
         int y = c;
-#pragma unroll
+#pragma unroll 1
         for (int o = 1; o < 32; o <<= 1) {
             const int z = __shfl_up_sync(0xffffffffu, y, o);
             if (lane >= o) y += z;
@@ -521,6 +514,7 @@ __global__ void __launch_bounds__(SEL1_THREADS)
     __syncthreads();
     if (tid < tiles * 32) cnt[tid] = wtot[wid] + x - mine;
     __syncthreads();
+#pragma unroll 1
     for (int u = 0; u < tiles; ++u) {
         const uint32_t b = __shfl_sync(0xffffffffu, bal, u);
         if ((mask >> u) & 1u)
@@ -532,7 +526,10 @@ __global__ void __launch_bounds__(SEL1_THREADS)
 cudaError_t select_launch(const StateDev& st, const SchedDev& sd, double t_end, cudaStream_t s)
 {
     if (st.n > 0 && st.n <= SEL1_MAX_N) {
-        select_one_cta_kernel<<<1, SEL1_THREADS, 0, s>>>(st.nkey, st.n, t_end, sd);
+        if (st.n <= 4 * SEL1_THREADS)
+            select_one_cta_kernel<4><<<1, SEL1_THREADS, 0, s>>>(st.nkey, st.n, t_end, sd);
+        else
+            select_one_cta_kernel<16><<<1, SEL1_THREADS, 0, s>>>(st.nkey, st.n, t_end, sd);
         return cudaGetLastError();
     }
     cudaError_t e = cudaMemsetAsync(sd.tmin_bits, 0xff, sizeof(unsigned long long), s);
