@@ -671,7 +671,7 @@ nb_status validate_idx(nb_ctx* c, int32_t n_act, const int32_t* idx)
 }
 
 // Whether a block step's select, prediction and force run in one launch: a
-// small system in HYBRID or DS with the default tile shapes.
+// small system in HYBRID with the default tile shapes.
 bool fused_step(const nb_ctx* c)
 {
     const nb_ctx::Variant &v0 = c->var[0], &v1 = c->var[1];

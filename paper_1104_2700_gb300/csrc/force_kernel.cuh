@@ -618,10 +618,8 @@ struct PolicyDS {
 
     using I = DSI;
     using Acc = DSAccs;
-    static constexpr bool HYB = false;
 
     __device__ static void load_i(const ForceParams& f, int p, int, I& s) { ds_load_i(f, p, s); }
-    __device__ static void limits_i(const ForceParams&, int, I&) {}
 
     template <bool MASK, int S>
     __device__ static void tile(const unsigned char* buf, int64_t j0, const Eps2& e2s,
@@ -739,7 +737,6 @@ struct PolicyHybrid {
 
     using I = HybridI;
     using Acc = HybridAcc;
-    static constexpr bool HYB = true;
 
     __device__ static void load_i(const ForceParams& f, int p, int particle, I& s)
     {

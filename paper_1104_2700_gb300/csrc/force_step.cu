@@ -1,17 +1,16 @@
 // Steps 1-4 of a block step of a small system in one launch: the next block
 // time and its block, the prediction, and the force on the block.
 //
-// At a few thousand particles a block step's kernels are latency: launches,
-// dependent loads, and above all instructions run once by a cold SM (~13
-// cycles each in straight-line code, where a warm one takes ~1.3).  Select and
-// predictor took 4 + 5.6 us of a ~29 us block step at N = 1024 beside a force
-// launch of ~10 us.  Here every CTA selects the block itself, and stages the j
-// tiles it sums by predicting them: a warp per component, in a loop over
-// 32-particle chunks, so that the code is short and fetched once.  A tile is
-// then summed by the CTA's four warps: near and double-single tiles a quarter
-// of the records each, a far tile (one FP32 run of 64) whole by one of them.
-// The price is the prediction done again for every i-group: ~10 % of summing a
-// tile, in launches that use a small part of the chip.
+// At a thousand particles a block step's kernels are latency: launches,
+// dependent loads, and instructions run once by a cold SM (~13 cycles each in
+// straight-line code, where a warm one takes ~1.3).  Beside a force launch of
+// ~10 us, select and predictor take 2.5 + 2.4 us of a 22.4 us block step.  Here
+// every CTA selects the block itself, and stages the j tiles it sums by
+// predicting them: a warp per component, in a loop over 32-particle chunks, so
+// that the code is short and fetched once.  A tile is then summed by the CTA's
+// four warps: a near tile a quarter of the records each, a far tile (one FP32
+// run of 64) whole by one of them.  The price is the select in every CTA and
+// the prediction again for every i-group; STEP_MAX_N says where that pays.
 #include <math_constants.h>
 
 #include "force_kernel.cuh"
@@ -130,7 +129,7 @@ __device__ __forceinline__ int step_select(const ForceParams& f, uint16_t* list,
 // Steps 2-3 of `chunks` chunks of 32 particles, particle_of(chunk, lane) (-1: a
 // ghost), into chunk % 2 of the tile at tile_of(chunk): the records of the
 // predictor kernel, bit for bit, with the tile's box after its second chunk.
-template <bool HYB, class P, class T>
+template <class P, class T>
 __device__ __forceinline__ void step_predict(const ForceParams& f, double t, int chunks,
                                              P particle_of, T tile_of)
 {
@@ -149,9 +148,8 @@ __device__ __forceinline__ void step_predict(const ForceParams& f, double t, int
         for (int e = 0; e < 5; ++e)
             if (e == 0 || c < 3) asm volatile("prefetch.global.L1 [%0];" ::"l"(p[e]));
     }
-    float qx = 0.f, iqx = 0.f, qv = 0.f, iqv = 0.f;
+    float qx, iqx;
     grid_quantum_f(st.bound[0], qx, iqx);
-    if (!HYB) grid_quantum_f(st.bound[1], qv, iqv);
     float lo_e = CUDART_INF_F, hi_e = -CUDART_INF_F;
 #pragma unroll 1
     for (int k = 0; k < chunks; ++k) {
@@ -172,16 +170,16 @@ __device__ __forceinline__ void step_predict(const ForceParams& f, double t, int
                 lo_e = fminf(lo_e, hi), hi_e = fmaxf(hi_e, hi);
             }
             float vh, vl;
-            split_velocity<HYB>(v, qv, iqv, vh, vl);
+            split_velocity<true>(v, 0.f, 0.f, vh, vl);
             A[c] = hi, B[c] = lo, C[c] = vh, D[c] = vl;
         } else {
             const Dsf gm = i >= 0 ? dsf_mass(f.G, st.m[i]) : Dsf{0.f, 0.f};
             const float g = cbrtf(gm.hi);
             A[3] = gm.hi, B[3] = gm.lo, C[3] = g * g;
-            if (!HYB || lane >= 8 || (k & 1)) D[3] = 0.f;
+            if (lane >= 8 || (k & 1)) D[3] = 0.f;
             lo_e = fminf(lo_e, -gm.hi), hi_e = fmaxf(hi_e, g * g);
         }
-        if (HYB && (k & 1)) {
+        if (k & 1) {
 #pragma unroll 1
             for (int o = 16; o > 0; o >>= 1) {
                 lo_e = fminf(lo_e, __shfl_xor_sync(0xffffffffu, lo_e, o));
@@ -234,7 +232,7 @@ __global__ void __launch_bounds__(ST_THREADS, K::MIN_CTAS) step_force_kernel(con
             // j tile of the walk's rank b0 + b; chunk 2 nb: the i particles
             auto jtile = [&](int b) { return static_cast<int>(tile_at(gi, b0 + b)); };
             __syncthreads();  // the last use of the staged tiles is over
-            step_predict<K::HYB>(
+            step_predict(
                 f, t_now, 2 * nb + (first ? 1 : 0),
                 [&](int k, int l) {
                     if (k == 2 * nb) return l < acts ? static_cast<int>(list[act0 + l]) : -1;
@@ -257,8 +255,7 @@ __global__ void __launch_bounds__(ST_THREADS, K::MIN_CTAS) step_force_kernel(con
                     s.vxh = s.vyh = s.vzh = s.vxl = s.vyl = s.vzl = 0.f;
                 }
                 K::limits_i(f, s.p, s);
-                if constexpr (K::GUARDED)
-                    guard_any = __any_sync(0xffffffffu, K::guarded(s));
+                guard_any = __any_sync(0xffffffffu, K::guarded(s));
             }
             if (g == 0) {  // the layout in global memory, as the predictor leaves it
                 const void* jl[4] = {f.jl0, f.jl1, f.jl2, f.jl3};
@@ -277,36 +274,30 @@ __global__ void __launch_bounds__(ST_THREADS, K::MIN_CTAS) step_force_kernel(con
                 const bool mask_self =
                     __any_sync(0xffffffffu, is[0].p >= j0 && is[0].p < j0 + TJ);
                 const int u0 = wib * (TJ / ST_WARPS), u1 = u0 + TJ / ST_WARPS;
-                if constexpr (K::GUARDED) {
-                    bool far = !mask_self && !guard_any;
-                    if (far) far = __all_sync(0xffffffffu, K::tile_far(buf, is[0], gi.e2.h));
-                    if (far) {
-                        if (((b0 + b) & 3) == wib) K::template far_tile<1>(buf, gi.e2, is, ac, 0);
-                        continue;
-                    }
-                    uint32_t nlo[1], nhi[1];
-                    if (guard_any) {
-                        if (mask_self)
-                            K::template tile<true, true, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1, nlo,
-                                                            nhi);
-                        else
-                            K::template tile<false, true, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1,
-                                                             nlo, nhi);
-                    } else {
-                        if (mask_self)
-                            K::template tile<true, false, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1,
-                                                             nlo, nhi);
-                        else
-                            K::template tile<false, false, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1,
-                                                              nlo, nhi);
-                    }
-                    K::template near_pass<1>(buf, gi.e2, is, ac, lane, nlo, nhi,
-                                             reinterpret_cast<float2*>(smem + wib * M::WARP +
-                                                                       WarpSmem<K>::BAR_BYTES));
-                } else {
-                    if (mask_self) K::template tile<true, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1);
-                    else K::template tile<false, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1);
+                bool far = !mask_self && !guard_any;
+                if (far) far = __all_sync(0xffffffffu, K::tile_far(buf, is[0], gi.e2.h));
+                if (far) {
+                    if (((b0 + b) & 3) == wib) K::template far_tile<1>(buf, gi.e2, is, ac, 0);
+                    continue;
                 }
+                uint32_t nlo[1], nhi[1];
+                if (guard_any) {
+                    if (mask_self)
+                        K::template tile<true, true, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1, nlo, nhi);
+                    else
+                        K::template tile<false, true, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1, nlo,
+                                                         nhi);
+                } else {
+                    if (mask_self)
+                        K::template tile<true, false, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1, nlo,
+                                                         nhi);
+                    else
+                        K::template tile<false, false, 1>(buf, j0, gi.e2, is, ac, 0, u0, u1, nlo,
+                                                          nhi);
+                }
+                K::template near_pass<1>(buf, gi.e2, is, ac, lane, nlo, nhi,
+                                         reinterpret_cast<float2*>(smem + wib * M::WARP +
+                                                                   WarpSmem<K>::BAR_BYTES));
             }
         }
         // (cta_finish starts with a barrier after its own area's stores; the
@@ -326,7 +317,6 @@ const void* step_k()
 const void* step_kernel_ptr(Prec p)
 {
     switch (p) {
-    case Prec::DS: return step_k<PolicyDS<1>>();
     case Prec::HYBRID: return step_k<PolicyHybrid<1>>();
     case Prec::HYBRID_SPJ: return step_k<PolicyHybrid<1, true>>();
     default: return nullptr;
@@ -335,7 +325,7 @@ const void* step_kernel_ptr(Prec p)
 
 size_t step_smem_bytes(Prec p)
 {
-    return p == Prec::DS ? StepSmem<PolicyDS<1>>::BYTES : StepSmem<PolicyHybrid<1>>::BYTES;
+    return step_kernel_ptr(p) ? StepSmem<PolicyHybrid<1>>::BYTES : 0;
 }
 
 }  // namespace nb

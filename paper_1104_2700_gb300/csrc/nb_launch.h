@@ -172,8 +172,8 @@ struct ForceArgs {
     // CTA by CTA (shared memory, then one global level) instead of by the
     // warp tree.
     int32_t cta_mode = 0;
-    // One system of at most STEP_MAX_N particles, HYBRID or DS, one i per
-    // lane, no j split: steps 1-4 of a block step to t_end in this launch,
+    // One system of at most STEP_MAX_N particles, HYBRID, one i per lane, no
+    // j split: steps 1-4 of a block step to t_end in this launch,
     // from the state st; the block and its time go to sd.
     bool fused = false;
     StateDev st;
@@ -189,7 +189,12 @@ struct ForceArgs {
     int32_t dyn_chunks = 0;
 };
 
-constexpr int STEP_MAX_N = 4096;
+// Largest system whose block steps take the one-launch kernel of force_step.cu:
+// N = 256 19.9 against 20.4 us a block step, 1024 21.1 against 22.4, 2048 23.6
+// against 23.7, 4096 28.5 against 26.7 (every CTA reads all the next-time keys,
+// and each i-group predicts every tile again).  HYBRID only: in DS it gains
+// nothing at any size (1024: 20.5 against 20.6, 2048: 23.6 against 21.7).
+constexpr int STEP_MAX_N = 1536;
 bool force_step_exists(Prec p);
 cudaError_t force_setup(Prec p, int it, int split);  // one-time attribute setup
 int force_ctas_per_sm(Prec p, int it, int split);
