@@ -70,7 +70,7 @@ struct nb_ctx {
     int64_t counter_stride = 0;
     int64_t counter_words = 0;
     uint32_t* status_dev = nullptr;
-    unsigned long long* ctr64 = nullptr;  // [0] block steps, [1] interactions
+    unsigned long long* ctr64 = nullptr;  // [0] block steps, [1] interactions, [2] t_end_dev
     double* energy_partials = nullptr;
     double* energy_out = nullptr;
     uint32_t* energy_ticket = nullptr;
@@ -87,9 +87,10 @@ struct nb_ctx {
     bool loaded = false;
     nb_status sticky = NB_OK;
     std::string err;
-    // CUDA graph of GRAPH_STEPS device-resident block steps for one t_end.
+    // CUDA graph of GRAPH_STEPS device-resident block steps to the time in
+    // t_end_dev.
     cudaGraphExec_t step_graph = nullptr;
-    double graph_t_end = 0.0;
+    double* t_end_dev = nullptr;
     // The particles are stored in a spatial order: internal index k holds the
     // caller's particle perm[k] (inv is the inverse).  For one system the
     // order follows a Morton curve through its bounding box, so the j tiles
@@ -679,7 +680,7 @@ bool fused_step(const nb_ctx* c)
            v0.split == 1 && v1.it == 1 && v1.split == 1 && c->j_parts == 1;
 }
 
-nb_status block_step(nb_ctx* c, double t_end)
+nb_status block_step(nb_ctx* c, nb::TimeLimit t_end)
 {
     const nb::ClusterDev* cl = c->ens ? &c->cl : nullptr;
     const unsigned long long* tkeys = c->ens ? c->cl.tkey : c->sd.tmin_bits;
@@ -729,15 +730,16 @@ nb_status block_step(nb_ctx* c, double t_end)
     return NB_OK;
 }
 
-// Capture GRAPH_STEPS block steps for t_end into c->step_graph.  Every node
-// reads its block (t_next, n_act, idx) from device memory, so one graph
-// serves every replay until t_end changes or the buffers are reallocated.
-nb_status build_step_graph(nb_ctx* c, double t_end)
+// Capture GRAPH_STEPS block steps into c->step_graph.  Every node reads its
+// block (t_next, n_act, idx) and the end time from device memory, so one graph
+// serves every call until the shapes or the buffers change (capturing and
+// instantiating it takes ~350 us, ~17 block steps of a small system).
+nb_status build_step_graph(nb_ctx* c)
 {
     drop_graph(c);
     NB_CK(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     nb_status s = NB_OK;
-    for (int k = 0; k < GRAPH_STEPS && s == NB_OK; ++k) s = block_step(c, t_end);
+    for (int k = 0; k < GRAPH_STEPS && s == NB_OK; ++k) s = block_step(c, {0.0, c->t_end_dev});
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
     if (s != NB_OK) {
@@ -751,7 +753,6 @@ nb_status build_step_graph(nb_ctx* c, double t_end)
         c->step_graph = nullptr;
         return fail(c, NB_ECUDA, "graph instantiate: %s", cudaGetErrorString(ei));
     }
-    c->graph_t_end = t_end;
     return NB_OK;
 }
 
@@ -905,8 +906,9 @@ nb_status nb_create(const nb_config* cfg, nb_ctx** out)
     if (cudaMemset(c->status_dev, 0, sizeof(uint32_t)) != cudaSuccess) return bail(NB_ECUDA);
     if (cudaMalloc(&c->st.bound, 2 * sizeof(uint32_t)) != cudaSuccess) return bail(NB_ENOMEM);
     if (cudaMemset(c->st.bound, 0, 2 * sizeof(uint32_t)) != cudaSuccess) return bail(NB_ECUDA);
-    if (cudaMalloc(&c->ctr64, 2 * sizeof(unsigned long long)) != cudaSuccess) return bail(NB_ENOMEM);
-    if (cudaMemset(c->ctr64, 0, 2 * sizeof(unsigned long long)) != cudaSuccess) return bail(NB_ECUDA);
+    if (cudaMalloc(&c->ctr64, 3 * sizeof(unsigned long long)) != cudaSuccess) return bail(NB_ENOMEM);
+    if (cudaMemset(c->ctr64, 0, 3 * sizeof(unsigned long long)) != cudaSuccess) return bail(NB_ECUDA);
+    c->t_end_dev = reinterpret_cast<double*>(c->ctr64 + 2);
     if (cudaMallocHost(&c->pinned, PINNED_BYTES) != cudaSuccess) return bail(NB_ENOMEM);
     *out = c;
     return NB_OK;
@@ -1104,7 +1106,7 @@ nb_status nb_select(nb_ctx* c, double t_end, double* t_next, int32_t* n_act, int
     unsigned long long* hk = reinterpret_cast<unsigned long long*>(c->pinned + 16);
     int32_t* hn = reinterpret_cast<int32_t*>(c->pinned + 24);
     if (c->ens) {
-        NB_CK(c, nb::cluster_select_launch(c->st, c->cl, c->sd, t_end, c->stream));
+        NB_CK(c, nb::cluster_select_launch(c->st, c->cl, c->sd, {t_end, nullptr}, c->stream));
         std::vector<unsigned long long> keys(c->cl.k);
         NB_CK(c, cudaMemcpyAsync(keys.data(), c->cl.tkey, keys.size() * sizeof(unsigned long long),
                                  cudaMemcpyDeviceToHost, c->stream));
@@ -1112,7 +1114,7 @@ nb_status nb_select(nb_ctx* c, double t_end, double* t_next, int32_t* n_act, int
         NB_CK(c, cudaStreamSynchronize(c->stream));
         *hk = *std::min_element(keys.begin(), keys.end());  // keys order like times
     } else {
-        NB_CK(c, nb::select_launch(c->st, c->sd, t_end, c->stream));
+        NB_CK(c, nb::select_launch(c->st, c->sd, {t_end, nullptr}, c->stream));
         NB_CK(c, cudaMemcpyAsync(hk, c->sd.tmin_bits, sizeof(*hk), cudaMemcpyDeviceToHost, c->stream));
         NB_CK(c, cudaMemcpyAsync(hn, c->sd.n_act, sizeof(*hn), cudaMemcpyDeviceToHost, c->stream));
         NB_CK(c, cudaStreamSynchronize(c->stream));
@@ -1265,7 +1267,7 @@ nb_status nb_block_step(nb_ctx* c, double t_end)
 {
     nb_status s = enter(c, true);
     if (s != NB_OK) return s;
-    return block_step(c, t_end);
+    return block_step(c, {t_end, nullptr});
 }
 
 nb_status nb_step_until(nb_ctx* c, double t_end, uint64_t* n_steps, uint64_t* n_interactions)
@@ -1277,11 +1279,14 @@ nb_status nb_step_until(nb_ctx* c, double t_end, uint64_t* n_steps, uint64_t* n_
     // run resumed from a checkpoint gets the order the original had)
     if ((s = refresh_order(c)) != NB_OK) return s;
     NB_CK(c, cudaMemsetAsync(c->ctr64, 0, 2 * sizeof(unsigned long long), c->stream));
-    if (!c->step_graph || c->graph_t_end != t_end) {
-        if ((s = build_step_graph(c, t_end)) != NB_OK) return s;
-    }
+    double* hte = reinterpret_cast<double*>(c->pinned + 80);
+    *hte = t_end;  // (no copy from it is in flight: every call ends synchronised)
+    NB_CK(c, cudaMemcpyAsync(c->t_end_dev, hte, sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    if (!c->step_graph && (s = build_step_graph(c)) != NB_OK) return s;
     int32_t* hn = reinterpret_cast<int32_t*>(c->pinned + 24);
     uint32_t* hs = reinterpret_cast<uint32_t*>(c->pinned + 28);
+    c->last_force_n_act = -1;
+    c->order_fresh = false;  // the positions move
     // Replay GRAPH_STEPS block steps at a time; once t_next passes t_end the
     // remaining steps of a replay are empty.  One host round trip per replay.
     for (;;) {

@@ -86,7 +86,8 @@ struct ForceParams {
     // step_force_kernel (force_step.cu) only: the state, G, the end of the
     // integration, and where the block it selects is published.
     StateDev st;
-    double G, t_end;
+    double G;
+    TimeLimit t_end;
     int32_t* sel_idx;
     int32_t* sel_n_act;
     unsigned long long* sel_tmin;

@@ -53,6 +53,7 @@ __device__ __forceinline__ int step_select(const ForceParams& f, uint16_t* list,
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int n = static_cast<int>(f.n);
     const int rows = (n + ST_THREADS - 1) / ST_THREADS;
+    const double t_end = f.t_end.get();
     unsigned long long best = ~0ull;
     uint32_t mask = 0u;
 #pragma unroll 1
@@ -81,7 +82,7 @@ __device__ __forceinline__ int step_select(const ForceParams& f, uint16_t* list,
 #pragma unroll
     for (int w = 1; w < ST_WARPS; ++w) low = wmin[w] < low ? wmin[w] : low;
     key = low;
-    if (best != low || !(dkey_decode(low) <= f.t_end)) mask = 0u;
+    if (best != low || !(dkey_decode(low) <= t_end)) mask = 0u;
     uint32_t bal = 0u;  // lane u: the warp's ballot of row u
 #pragma unroll 1
     for (int u = 0; u < rows; ++u) {

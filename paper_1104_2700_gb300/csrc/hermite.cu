@@ -362,9 +362,10 @@ __device__ int block_exclusive_scan(int v, int* total)
 
 __global__ void __launch_bounds__(SCHED_THREADS)
     count_kernel(const unsigned long long* __restrict__ nkey, int64_t n,
-                 const unsigned long long* tkeys, const int32_t* cluster_of, double t_end,
+                 const unsigned long long* tkeys, const int32_t* cluster_of, TimeLimit limit,
                  SchedDev sd)
 {
+    const double t_end = limit.get();
     int c = 0;
     const int64_t base = (int64_t)blockIdx.x * SCHED_CHUNK + (int64_t)threadIdx.x * SCHED_PER_THREAD;
 #pragma unroll
@@ -402,9 +403,10 @@ __global__ void __launch_bounds__(SCHED_THREADS)
 
 __global__ void __launch_bounds__(SCHED_THREADS)
     scatter_kernel(const unsigned long long* __restrict__ nkey, int64_t n,
-                   const unsigned long long* tkeys, const int32_t* cluster_of, double t_end,
+                   const unsigned long long* tkeys, const int32_t* cluster_of, TimeLimit limit,
                    SchedDev sd)
 {
+    const double t_end = limit.get();
     const int64_t base = (int64_t)blockIdx.x * SCHED_CHUNK + (int64_t)threadIdx.x * SCHED_PER_THREAD;
     unsigned flags = 0;
     int c = 0;
@@ -447,11 +449,12 @@ __device__ __forceinline__ unsigned long long warp_min_key(unsigned long long k)
 // cold SM pays for every instruction of it).
 template <int BATCH>
 __global__ void __launch_bounds__(SEL1_THREADS)
-    select_one_cta_kernel(const unsigned long long* __restrict__ nkey, int64_t n, double t_end,
+    select_one_cta_kernel(const unsigned long long* __restrict__ nkey, int64_t n, TimeLimit limit,
                           SchedDev sd)
 {
     __shared__ unsigned long long wmin[SEL1_THREADS / 32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const double t_end = limit.get();
     unsigned long long best = ~0ull;
     uint32_t mask = 0u;
     const int tiles = static_cast<int>((n + SEL1_THREADS - 1) / SEL1_THREADS);  // <= 32
@@ -523,7 +526,7 @@ __global__ void __launch_bounds__(SEL1_THREADS)
     }
 }
 
-cudaError_t select_launch(const StateDev& st, const SchedDev& sd, double t_end, cudaStream_t s)
+cudaError_t select_launch(const StateDev& st, const SchedDev& sd, TimeLimit t_end, cudaStream_t s)
 {
     if (st.n > 0 && st.n <= SEL1_MAX_N) {
         if (st.n <= 4 * SEL1_THREADS)
@@ -561,9 +564,10 @@ __device__ __forceinline__ void min_count_merge(unsigned long long& best, int& n
 
 __global__ void cluster_tmin_kernel(const unsigned long long* __restrict__ nkey,
                                     const int64_t* off, unsigned long long* tkey, int32_t* cnt,
-                                    double t_end)
+                                    TimeLimit limit)
 {
     const int c = blockIdx.x;
+    const double t_end = limit.get();
     unsigned long long best = ~0ull;
     int n = 0;
     for (int64_t i = off[c] + threadIdx.x; i < off[c + 1]; i += blockDim.x)
@@ -597,7 +601,7 @@ __global__ void cluster_tmin_kernel(const unsigned long long* __restrict__ nkey,
 }
 
 cudaError_t cluster_select_launch(const StateDev& st, const ClusterDev& cl, const SchedDev& sd,
-                                  double t_end, cudaStream_t s)
+                                  TimeLimit t_end, cudaStream_t s)
 {
     if (st.n <= 0 || cl.k <= 0) return cudaMemsetAsync(sd.n_act, 0, sizeof(int32_t), s);
     const int64_t nb64 = (st.n + SCHED_CHUNK - 1) / SCHED_CHUNK;

@@ -28,6 +28,16 @@ enum class Prec : int {
 inline bool is_mixed(Prec p) { return p == Prec::MIXED || p == Prec::MIXED_SPJ; }
 inline bool is_hybrid(Prec p) { return p == Prec::HYBRID || p == Prec::HYBRID_SPJ; }
 
+// The time past which no block is due: a value, or a double in device memory,
+// so that a captured graph of block steps serves every end time.
+struct TimeLimit {
+    double value = 0.0;
+    const double* dev = nullptr;
+#ifdef __CUDACC__
+    __device__ __forceinline__ double get() const { return dev ? __ldcg(dev) : value; }
+#endif
+};
+
 // Device Hermite state of one context, structure of arrays.  x, v, a, j
 // hold 3*n doubles: component c of particle i at [c*n + i].
 struct StateDev {
@@ -178,7 +188,8 @@ struct ForceArgs {
     bool fused = false;
     StateDev st;
     SchedDev sd;
-    double G = 1.0, t_end = 0.0;
+    double G = 1.0;
+    TimeLimit t_end;
     // n_act known at launch (>= 0): the kernel does not read n_act_dev.
     int32_t n_act_host = -1;
     // Optional: idx holds caller indices, idx_map[i] is the layout slot of i.
@@ -220,7 +231,7 @@ cudaError_t predict_launch(const StateDev& st, Prec p, const JLayout& jl, double
 // Ensemble step 1 (per-cluster next times, then one global compaction) and
 // the force plan of the active list (idx ascending, clusters contiguous).
 cudaError_t cluster_select_launch(const StateDev& st, const ClusterDev& cl, const SchedDev& sd,
-                                  double t_end, cudaStream_t s);
+                                  TimeLimit t_end, cudaStream_t s);
 // With from_counts the plan takes each cluster's share of the (sorted) active
 // list from cl.cnt, written by the select of the same block step; otherwise
 // it finds the shares in idx by binary search (any sorted list).
@@ -238,7 +249,7 @@ double time_from_key(unsigned long long k);
 
 // Step 1: t_next = min(t + dt), stable compaction of the active block.
 // When t_next > t_end the block is empty (n_act = 0).
-cudaError_t select_launch(const StateDev& st, const SchedDev& sd, double t_end,
+cudaError_t select_launch(const StateDev& st, const SchedDev& sd, TimeLimit t_end,
                           cudaStream_t s);
 
 // Steps 5-8 on the active list at the time in *t_bits.
