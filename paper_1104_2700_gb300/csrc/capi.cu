@@ -685,6 +685,7 @@ nb_status block_step(nb_ctx* c, nb::TimeLimit t_end)
     const nb::ClusterDev* cl = c->ens ? &c->cl : nullptr;
     const unsigned long long* tkeys = c->ens ? c->cl.tkey : c->sd.tmin_bits;
     const bool fused = fused_step(c);
+    bool planned = false;  // ensemble: the select has written the force plan too
     if (fused) {
         nb::ForceArgs f = force_args(c, c->prec, c->jl, c->sd.idx, c->sd.n_act);
         f.grid = c->var[0].grid;
@@ -696,13 +697,16 @@ nb_status block_step(nb_ctx* c, nb::TimeLimit t_end)
         f.t_end = t_end;
         NB_CK(c, nb::force_launch(f, c->stream));
     } else if (c->ens)
-        NB_CK(c, nb::cluster_select_launch(c->st, c->cl, c->sd, t_end, c->stream));
+        NB_CK(c, nb::cluster_select_launch(c->st, c->cl, c->sd, t_end, c->stream,
+                                           32 * c->var[0].it / c->var[0].split, &planned));
     else
         NB_CK(c, nb::select_launch(c->st, c->sd, t_end, c->stream));
     if (!fused) {
         NB_CK(c, nb::predict_launch(c->st, c->prec, c->jl, c->cfg.G, tkeys, 0.0, c->sd.n_act,
                                     c->stream, cl));
-        const nb_status s = run_force_list(c, c->prec, c->jl, c->sd.idx, c->sd.n_act, -1, true);
+        const nb_status s =
+            planned ? run_force(c, c->prec, c->jl, c->sd.idx, c->sd.n_act)
+                    : run_force_list(c, c->prec, c->jl, c->sd.idx, c->sd.n_act, -1, true);
         if (s != NB_OK) return s;
     }
     nb::CorrectArgs ca;

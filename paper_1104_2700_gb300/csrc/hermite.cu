@@ -549,65 +549,184 @@ cudaError_t select_launch(const StateDev& st, const SchedDev& sd, TimeLimit t_en
 }
 
 // Ensemble step 1: block c finds the next time of cluster c and how many of
-// its particles reach it (0 when that time lies past t_end): a reduction of
-// (smallest key, count of that key) pairs.
-__device__ __forceinline__ void min_count_merge(unsigned long long& best, int& n,
-                                                unsigned long long ob, int on)
+// its particles reach it (0 when that time lies past t_end).
+constexpr int CLS_THREADS = 256;
+
+__global__ void __launch_bounds__(CLS_THREADS)
+    cluster_tmin_kernel(const unsigned long long* __restrict__ nkey, const int64_t* off,
+                        unsigned long long* tkey, int32_t* cnt, TimeLimit limit)
 {
-    if (ob < best) {
-        best = ob;
-        n = on;
-    } else if (ob == best) {
-        n += on;
+    const int c = blockIdx.x;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const double t_end = limit.get();
+    const int64_t end = off[c + 1];
+    unsigned long long best = ~0ull;
+    int n = 0;
+#pragma unroll 1
+    for (int64_t i0 = off[c] + threadIdx.x; i0 < end; i0 += 8 * CLS_THREADS) {
+        unsigned long long kk[8];  // one round trip
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            const int64_t i = i0 + v * CLS_THREADS;
+            kk[v] = i < end ? __ldcg(nkey + i) : ~0ull;
+        }
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            if (kk[v] < best) best = kk[v], n = 0;
+            n += kk[v] == best;
+        }
+    }
+    __shared__ unsigned long long wbest[CLS_THREADS / 32];
+    __shared__ int wn[CLS_THREADS / 32];
+    const unsigned long long wlow = warp_min_key(best);
+    n = __reduce_add_sync(0xffffffffu, best == wlow ? n : 0);
+    if (lane == 0) wbest[wid] = wlow, wn[wid] = n;
+    __syncthreads();
+    if (wid == 0) {
+        const bool have = lane < CLS_THREADS / 32;
+        best = have ? wbest[lane] : ~0ull;
+        const unsigned long long low = warp_min_key(best);
+        n = __reduce_add_sync(0xffffffffu, have && best == low ? wn[lane] : 0);
+        if (lane == 0) {
+            tkey[c] = low;
+            cnt[c] = (low != ~0ull && dkey_decode(low) <= t_end) ? n : 0;
+        }
     }
 }
 
-__global__ void cluster_tmin_kernel(const unsigned long long* __restrict__ nkey,
-                                    const int64_t* off, unsigned long long* tkey, int32_t* cnt,
-                                    TimeLimit limit)
+// Sum over the block, of three counts.
+struct Sum3 {
+    int a, b;
+    int64_t t;
+};
+__device__ __forceinline__ Sum3 block_sum3(Sum3 v)
+{
+    __shared__ Sum3 w[CLS_THREADS / 32];
+    const int lane = threadIdx.x & 31;
+    v.a = __reduce_add_sync(0xffffffffu, v.a);
+    v.b = __reduce_add_sync(0xffffffffu, v.b);
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) v.t += __shfl_xor_sync(0xffffffffu, v.t, o);
+    if (lane == 0) w[threadIdx.x >> 5] = v;
+    __syncthreads();
+    Sum3 s = {0, 0, 0};
+#pragma unroll 1
+    for (int k = 0; k < CLS_THREADS / 32; ++k) s.a += w[k].a, s.b += w[k].b, s.t += w[k].t;
+    return s;
+}
+
+// The block of an ensemble and its force plan from the clusters' next times and
+// counts: block c sums the counts of the clusters before it, writes its own
+// members, ascending, and (gi > 0) cuts them into i-groups of at most gi laid
+// after the earlier clusters'.  In place of a count, a scatter and a one-CTA
+// plan launch: every block reads every earlier count, so for ensembles of at
+// most CLS_MAX systems.  256 rows of particles a pass, as in the one-CTA select.
+constexpr int CLS_MAX = 4096;
+
+__global__ void __launch_bounds__(CLS_THREADS)
+    cluster_block_kernel(const unsigned long long* __restrict__ nkey, const ClusterDev cl,
+                         SchedDev sd, int gi)
 {
     const int c = blockIdx.x;
-    const double t_end = limit.get();
-    unsigned long long best = ~0ull;
-    int n = 0;
-    for (int64_t i = off[c] + threadIdx.x; i < off[c + 1]; i += blockDim.x)
-        min_count_merge(best, n, nkey[i], 1);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int on = __shfl_xor_sync(0xffffffffu, n, o);
-        min_count_merge(best, n, ob, on);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    auto groups = [&](int n) { return gi > 0 ? (n + gi - 1) / gi : 0; };
+    auto tiles = [&](int q) { return (cl.joff[q + 1] - cl.joff[q]) / TJ; };
+    Sum3 v = {0, 0, 0};
+    for (int q = tid; q < c; q += CLS_THREADS) {
+        const int n = cl.cnt[q], g = groups(n);
+        v.a += n;
+        v.b += g;
+        if (g) v.t += g * tiles(q);
     }
-    __shared__ unsigned long long wbest[32];
-    __shared__ int wn[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) wbest[wid] = best, wn[wid] = n;
-    __syncthreads();
-    if (wid == 0) {
-        const bool have = lane < (int)(blockDim.x >> 5);
-        best = have ? wbest[lane] : ~0ull;
-        n = have ? wn[lane] : 0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-            const int on = __shfl_xor_sync(0xffffffffu, n, o);
-            min_count_merge(best, n, ob, on);
+    const Sum3 base = block_sum3(v);
+    const int n = cl.cnt[c], g = groups(n);
+    const int64_t nt = tiles(c);
+    if (gi > 0 && base.b + g <= cl.max_groups) {  // (always, as the plan is sized)
+        for (int k = tid; k < g; k += CLS_THREADS) {
+            cl.grp_cluster[base.b + k] = c;
+            cl.grp_act_begin[base.b + k] = base.a + k * gi;
+            cl.grp_act_count[base.b + k] = n - k * gi < gi ? n - k * gi : gi;
+            cl.grp_tile0[base.b + k] = base.t + k * nt;
         }
-        if (lane == 0) {
-            tkey[c] = best;
-            cnt[c] = (best != ~0ull && dkey_decode(best) <= t_end) ? n : 0;
+    }
+    if (c == cl.k - 1 && tid == 0) {
+        *sd.n_act = base.a + n;
+        if (gi > 0) {
+            cl.grp_tile0[base.b + g] = base.t + g * nt;
+            cl.plan_scalars[0] = base.b + g;
+            cl.plan_scalars[1] = base.t + g * nt;
+        }
+    }
+    if (n == 0) return;
+    const unsigned long long key = cl.tkey[c];
+    constexpr int W = CLS_THREADS / 32, ROWS = 32;
+    __shared__ int cnt[ROWS * W];  // entry (row u, warp w)
+    __shared__ int wtot[W];
+    const int64_t end = cl.off[c + 1];
+    int at = base.a;
+    for (int64_t i0 = cl.off[c]; i0 < end; i0 += ROWS * CLS_THREADS) {
+        uint32_t mask = 0u, bal = 0u;
+#pragma unroll 1
+        for (int u0 = 0; u0 < ROWS && i0 + u0 * CLS_THREADS < end; u0 += 8) {
+            unsigned long long kk[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int64_t i = i0 + tid + (u0 + e) * CLS_THREADS;
+                kk[e] = i < end ? __ldcg(nkey + i) : ~key;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) mask |= static_cast<uint32_t>(kk[e] == key) << (u0 + e);
+        }
+#pragma unroll 1
+        for (int u = 0; u < ROWS; ++u) {
+            const uint32_t b = __ballot_sync(0xffffffffu, (mask >> u) & 1u);
+            if (lane == u) bal = b;
+        }
+        __syncthreads();  // the previous pass's reads of cnt
+        cnt[lane * W + wid] = __popc(bal);
+        __syncthreads();
+        const int mine = cnt[tid];  // ROWS * W == CLS_THREADS entries, one each
+        static_assert(ROWS * W == CLS_THREADS, "an entry per thread");
+        int x = mine;
+#pragma unroll 1
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wtot[wid] = x;
+        __syncthreads();
+        int before = at;
+#pragma unroll 1
+        for (int k = 0; k < W; ++k) {
+            before += k < wid ? wtot[k] : 0;
+            at += wtot[k];
+        }
+        cnt[tid] = before + x - mine;
+        __syncthreads();
+#pragma unroll 1
+        for (int u = 0; u < ROWS; ++u) {
+            const uint32_t b = __shfl_sync(0xffffffffu, bal, u);
+            if ((b >> lane) & 1u)
+                sd.idx[cnt[u * W + wid] + __popc(b & ((1u << lane) - 1u))] =
+                    static_cast<int32_t>(i0 + tid + u * CLS_THREADS);
         }
     }
 }
 
 cudaError_t cluster_select_launch(const StateDev& st, const ClusterDev& cl, const SchedDev& sd,
-                                  TimeLimit t_end, cudaStream_t s)
+                                  TimeLimit t_end, cudaStream_t s, int gi, bool* planned)
 {
+    if (planned) *planned = false;
     if (st.n <= 0 || cl.k <= 0) return cudaMemsetAsync(sd.n_act, 0, sizeof(int32_t), s);
+    cluster_tmin_kernel<<<cl.k, CLS_THREADS, 0, s>>>(st.nkey, cl.off, cl.tkey, cl.cnt, t_end);
+    if (cl.k <= CLS_MAX) {
+        cluster_block_kernel<<<cl.k, CLS_THREADS, 0, s>>>(st.nkey, cl, sd, gi);
+        if (planned) *planned = gi > 0;
+        return cudaGetLastError();
+    }
     const int64_t nb64 = (st.n + SCHED_CHUNK - 1) / SCHED_CHUNK;
     if (nb64 > sd.max_blocks) return cudaErrorInvalidValue;
     const int nb = static_cast<int>(nb64);
-    cluster_tmin_kernel<<<cl.k, 256, 0, s>>>(st.nkey, cl.off, cl.tkey, cl.cnt, t_end);
     count_kernel<<<nb, SCHED_THREADS, 0, s>>>(st.nkey, st.n, cl.tkey, cl.cluster_of, t_end, sd);
     scatter_kernel<<<nb, SCHED_THREADS, 0, s>>>(st.nkey, st.n, cl.tkey, cl.cluster_of, t_end, sd);
     return cudaGetLastError();

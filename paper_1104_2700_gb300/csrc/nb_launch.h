@@ -231,7 +231,8 @@ cudaError_t predict_launch(const StateDev& st, Prec p, const JLayout& jl, double
 // Ensemble step 1 (per-cluster next times, then one global compaction) and
 // the force plan of the active list (idx ascending, clusters contiguous).
 cudaError_t cluster_select_launch(const StateDev& st, const ClusterDev& cl, const SchedDev& sd,
-                                  TimeLimit t_end, cudaStream_t s);
+                                  TimeLimit t_end, cudaStream_t s, int gi = 0,
+                                  bool* planned = nullptr);
 // With from_counts the plan takes each cluster's share of the (sorted) active
 // list from cl.cnt, written by the select of the same block step; otherwise
 // it finds the shares in idx by binary search (any sorted list).

@@ -190,3 +190,24 @@ def test_hybrid_ensemble_integration_matches_oracle_per_system(gpu, orc):
         assert dr < 1e-6 and dv < 1e-5, report[-1]
         assert same_dt >= 0.95, report[-1]
     assert inter == pytest.approx(orc_inter, rel=0.05)
+
+
+@pytest.mark.parametrize("sizes", [[1, 2, 255, 256, 257, 8191, 8193, 3], [2] * 4097],
+                         ids=["edges", "many"])
+def test_block_lists_at_size_edges(gpu, sizes):
+    """The block lists of systems at the edges of the per-system pass (256
+    threads, 8192 particles a pass) and of more systems than it serves: each
+    system's members at its own next time, ascending, over several steps."""
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    parts = [ics.plummer(max(n, 2), 40 + q % 50) for q, n in enumerate(sizes)]
+    m, r, v = (np.concatenate([p[d][:n] for p, n in zip(parts, sizes)]) for d in range(3))
+    with gpu.Context("ds") as c:
+        c.set_ensemble(off, m, r, v, np.full(len(sizes), 0.05), 0.02)
+        for _ in range(4):
+            s = c.get_state()
+            nxt = s["t"] + s["dt"]
+            want = np.concatenate([a + np.flatnonzero(nxt[a:b] == nxt[a:b].min())
+                                   for a, b in zip(off[:-1], off[1:])])
+            t, idx = c.select()
+            assert t == nxt.min() and np.array_equal(idx, want)
+            c.block_step(1.0)
