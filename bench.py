@@ -707,7 +707,7 @@ def algorithmic_bytes(prec, n_j, n_act):
 # Kernels of one graph-replayed block step of the sweep (N = 16384): the
 # state roll-back (nb_restore), the one-CTA select (systems up to 32768
 # particles), predict, the two force launch variants (each returns at once
-# outside its n_act window), correct.
+# outside its n_act window; HYBRID keeps both at this size), correct.
 LAUNCHES_PER_BLOCK_STEP = 6
 DTYPES = {"ds": "f32x2 (double-single on the FP32 pipes)", "mixed": "f32", "fp64": "f64",
           "mixed_spj": "f32", "hybrid_spj": "f32 (far pairs) + f32x2 double-single (near pairs)",

@@ -133,8 +133,9 @@ void nb_config_init(nb_config* cfg);
  * whose block size the host knows (nb_force with n_act >= 0) on fewer than
  * tiny_split particles uses a third, "tiny" shape; a block step, whose size
  * is on the device, launches the small and the large shape as two parallel
- * branches (one returns at once) and never the tiny one, since a third
- * branch costs a block step more than the shape saves.  i_per_thread is the
+ * branches (one returns at once; or one launch where the two are the same)
+ * and never the tiny one, since a third branch costs a block step more than
+ * the shape saves.  i_per_thread is the
  * i-tile per lane; j_split the lanes that share one i, each taking every
  * j_split-th j of a tile (an i-group is 32 * i_per_thread / j_split
  * particles); ctas_per_sm sets the persistent grid, which fixes how far each
