@@ -371,11 +371,22 @@ nb_status check_status(nb_ctx* c)
 nb::ForceArgs force_args(nb_ctx* c, Prec p, const nb::JLayout& jl, const int32_t* idx,
                          const int32_t* n_act_dev);
 
+// A caller's device arrays for the results, written by the force kernel beside
+// the context's own (each may be null).
+struct Outputs {
+    double* acc = nullptr;
+    double* jerk = nullptr;
+    double* pot = nullptr;
+};
+
 nb_status run_force(nb_ctx* c, Prec p, const nb::JLayout& jl, const int32_t* idx,
                     const int32_t* n_act_dev, int32_t n_act_host = -1,
-                    const int32_t* idx_map = nullptr)
+                    const int32_t* idx_map = nullptr, const Outputs& out = Outputs())
 {
     nb::ForceArgs f = force_args(c, p, jl, idx, n_act_dev);
+    f.out_acc = out.acc;
+    f.out_jerk = out.jerk;
+    f.out_pot = out.pot;
     f.n_act_host = n_act_host;  // known here: the kernel need not read it
     f.idx_map = idx_map;
     if (p == c->prec && c->j_parts > 1) {
@@ -660,6 +671,21 @@ std::vector<int32_t> internal_sorted(const nb_ctx* c, int32_t n_act, const int32
     std::vector<int32_t> sorted(n_act);
     for (int32_t k = 0; k < n_act; ++k) sorted[k] = c->h_inv[idx[perm[k]]];
     return sorted;
+}
+
+// Whether a kernel of the context may write doubles at p: null (not written),
+// or aligned device memory of the context's device.  Anything else goes through
+// a copy, which reports what it cannot reach.
+bool on_this_device(const nb_ctx* c, const void* p)
+{
+    if (!p) return true;
+    if (reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0) return false;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == c->device;
 }
 
 nb_status validate_idx(nb_ctx* c, int32_t n_act, const int32_t* idx)
@@ -1150,6 +1176,7 @@ nb_status nb_force(nb_ctx* c, int32_t n_act, const int32_t* idx, double* acc, do
             if (idx[k] <= idx[k - 1])
                 return fail(c, NB_EINVAL, "ensemble force needs idx strictly ascending");
     std::vector<int32_t> perm;  // host list: entry k of the internal list is idx[perm[k]]
+    bool direct = false;        // the force kernel writes the caller's arrays itself
     if (n_act > 0 && !on_device) {
         if ((s = sync_host_order(c)) != NB_OK) return s;
         const std::vector<int32_t> sorted = internal_sorted(c, n_act, idx, perm);
@@ -1167,13 +1194,18 @@ nb_status nb_force(nb_ctx* c, int32_t n_act, const int32_t* idx, double* acc, do
             return s;
     } else if (n_act > 0) {
         // one launch: n_act as a parameter, and a device list in the caller's
-        // numbering mapped to layout slots by the kernel itself
+        // numbering mapped to layout slots by the kernel itself, which also
+        // writes the caller's arrays where they are this device's memory
+        Outputs out;
+        direct = on_device && on_this_device(c, acc) && on_this_device(c, jerk) &&
+                 on_this_device(c, pot);
+        if (direct) out = {acc, jerk, pot};
         if ((s = run_force(c, c->prec, c->jl, on_device ? idx : c->idx_user, c->n_act_user,
-                           n_act, on_device ? c->inv_dev : nullptr)) != NB_OK)
+                           n_act, on_device ? c->inv_dev : nullptr, out)) != NB_OK)
             return s;
     }
     c->last_force_n_act = n_act;
-    if (n_act > 0 && on_device) {
+    if (n_act > 0 && on_device && !direct) {
         const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
         if (acc) NB_CK(c, cudaMemcpyAsync(acc, c->acc1, 3 * (size_t)n_act * sizeof(double), k, c->stream));
         if (jerk) NB_CK(c, cudaMemcpyAsync(jerk, c->jerk1, 3 * (size_t)n_act * sizeof(double), k, c->stream));

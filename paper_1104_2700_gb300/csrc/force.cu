@@ -167,6 +167,9 @@ cudaError_t force_launch(const ForceArgs& a, cudaStream_t s)
     f.jerk = a.jerk;
     f.pot = a.pot;
     f.snap = a.snap;
+    f.out_acc = a.out_acc;
+    f.out_jerk = a.out_jerk;
+    f.out_pot = a.out_pot;
     f.scratch = a.scratch;
     f.counters = a.counters;
     f.counter_stride = a.counter_stride;

@@ -40,6 +40,11 @@ struct ForceParams {
     double* jerk;
     double* pot;
     double* snap;  // sixth-order variant: [n_act][3]
+    // a second destination of acc, jerk and pot (each may be null): the arrays
+    // of a caller on the device
+    double* out_acc;
+    double* out_jerk;
+    double* out_pot;
     double* scratch;
     uint32_t* counters;      // RLEVELS arrays of counter_stride entries
     int64_t counter_stride;  // >= warps + groups
@@ -1433,6 +1438,20 @@ struct ClusterPlan {
     }
 };
 
+// Row a of the results.
+__device__ __forceinline__ void write_row(const ForceParams& f, int64_t a, const double* o)
+{
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f.acc[3 * a + c] = o[c], f.jerk[3 * a + c] = o[3 + c];
+    f.pot[a] = o[6];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (f.out_acc) f.out_acc[3 * a + c] = o[c];
+        if (f.out_jerk) f.out_jerk[3 * a + c] = o[3 + c];
+    }
+    if (f.out_pot) f.out_pot[a] = o[6];
+}
+
 // CTA mode, after the tiles: this warp's sums (zeros if it had no tile) into
 // its own ring, which no copy uses any more; the four warps added in warp
 // order as the CTA's entry; the CTAs' entries of group cg added in a tree
@@ -1573,13 +1592,7 @@ __device__ __noinline__ void cta_finish(const ForceParams& f, unsigned char* sme
                 double o[NV];
 #pragma unroll
                 for (int c = 0; c < NV; ++c) o[c] = tree_value(fin[c * GI + q * IW + ir]);
-                f.acc[3 * a + 0] = o[0];
-                f.acc[3 * a + 1] = o[1];
-                f.acc[3 * a + 2] = o[2];
-                f.jerk[3 * a + 0] = o[3];
-                f.jerk[3 * a + 1] = o[4];
-                f.jerk[3 * a + 2] = o[5];
-                f.pot[a] = o[6];
+                write_row(f, a, o);
                 if constexpr (K::NV > 7) K::finish(f, is[q], a, o);
             }
         }
@@ -1968,13 +1981,7 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
                         double o[NV];
 #pragma unroll
                         for (int c = 0; c < NV; ++c) o[c] = tree_value(v[q][c]);
-                        f.acc[3 * a + 0] = o[0];
-                        f.acc[3 * a + 1] = o[1];
-                        f.acc[3 * a + 2] = o[2];
-                        f.jerk[3 * a + 0] = o[3];
-                        f.jerk[3 * a + 1] = o[4];
-                        f.jerk[3 * a + 2] = o[5];
-                        f.pot[a] = o[6];
+                        write_row(f, a, o);
                         if constexpr (K::NV > 7) K::finish(f, is[q], a, o);
                     }
                 }

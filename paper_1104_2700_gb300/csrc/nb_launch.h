@@ -157,6 +157,10 @@ struct ForceArgs {
     double* jerk = nullptr;  // [n_act][3]
     double* pot = nullptr;   // [n_act]
     double* snap = nullptr;  // [n_act][3], FP64_H6 only
+    // a second destination of the results (each may be null)
+    double* out_acc = nullptr;
+    double* out_jerk = nullptr;
+    double* out_pot = nullptr;
     double* scratch = nullptr;
     uint32_t* counters = nullptr;   // force_counter_entries() zeroed words
     int64_t counter_stride = 0;     // entries per reduction level
