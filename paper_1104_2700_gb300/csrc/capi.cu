@@ -46,6 +46,7 @@ struct nb_ctx {
         int it = 1;
         int grid = 0;
         int split = 1;  // lanes per i (j split inside a warp)
+        bool full = true;  // as many CTAs per SM as fit
     } var[3];
     int32_t nact_split = 1024;
     int32_t tiny_split = 0;
@@ -428,8 +429,14 @@ nb_status run_force(nb_ctx* c, Prec p, const nb::JLayout& jl, const int32_t* idx
     // are launched, the small one on the aux stream; exactly one of them does
     // any work, and neither touches memory the other uses before it has read
     // n_act.
-    NB_CK(c, cudaEventRecord(c->ev_fork, c->stream));
-    NB_CK(c, cudaStreamWaitEvent(c->aux, c->ev_fork, 0));
+    // A large variant that leaves room on the SMs would be placed around the
+    // idle one's CTAs, unevenly (N = 16384, every particle, 3 of 4 CTAs per SM:
+    // 687 us a block step against 547); it then runs after the small one.
+    const bool parallel = c->var[1].full;
+    if (parallel) {
+        NB_CK(c, cudaEventRecord(c->ev_fork, c->stream));
+        NB_CK(c, cudaStreamWaitEvent(c->aux, c->ev_fork, 0));
+    }
     for (int v = 0; v < 2; ++v) {
         f.it = c->var[v].it;
         f.split = c->var[v].split;
@@ -437,10 +444,12 @@ nb_status run_force(nb_ctx* c, Prec p, const nb::JLayout& jl, const int32_t* idx
         f.cta_mode = !c->ens && v == 0;  // small blocks: CTA-level sums
         f.nact_lo = v == 0 ? 0 : c->nact_split;
         f.nact_hi = v == 0 ? c->nact_split : 0x7fffffff;
-        NB_CK(c, nb::force_launch(f, v == 0 ? c->aux : c->stream));
+        NB_CK(c, nb::force_launch(f, v == 0 && parallel ? c->aux : c->stream));
     }
-    NB_CK(c, cudaEventRecord(c->ev_join, c->aux));
-    NB_CK(c, cudaStreamWaitEvent(c->stream, c->ev_join, 0));
+    if (parallel) {
+        NB_CK(c, cudaEventRecord(c->ev_join, c->aux));
+        NB_CK(c, cudaStreamWaitEvent(c->stream, c->ev_join, 0));
+    }
     return NB_OK;
 }
 
@@ -926,6 +935,7 @@ nb_status nb_create(const nb_config* cfg, nb_ctx** out)
         c->var[v].it = it;
         c->var[v].split = split;
         c->var[v].grid = per_sm * c->num_sms;
+        c->var[v].full = per_sm >= occ;
     }
     c->var[2] = c->var[0];  // no tiny variant until nb_autotune or nb_set_tuning sets one
     if (nb::force_setup(Prec::FP64, 1, 1) != cudaSuccess) return bail(NB_ECUDA);
@@ -1686,6 +1696,8 @@ nb_status nb_autotune(nb_ctx* c, nb_tuning* out)
     c->var[1] = {best[1]->it, best[1]->cps * c->num_sms, best[1]->split};
     c->var[2] = best[2] ? nb_ctx::Variant{best[2]->it, best[2]->cps * c->num_sms, best[2]->split}
                         : c->var[0];
+    c->var[1].full =
+        best[1]->cps >= nb::force_ctas_per_sm(c->prec, best[1]->it, best[1]->split);
     c->nact_split = split_probe == 3 ? 1024 : 4096;
     c->tiny_split = tiny_probe == 0 ? 0 : tiny_probe == 1 ? 64 : 160;
     drop_graph(c);
@@ -1748,6 +1760,7 @@ nb_status nb_set_tuning(nb_ctx* c, const nb_tuning* t)
         const Shape& q = sh[v == 2 && t->tiny_split == 0 ? 0 : v];
         c->var[v] = {q.it, q.cps * c->num_sms, q.split};
     }
+    c->var[1].full = sh[1].cps >= nb::force_ctas_per_sm(c->prec, sh[1].it, sh[1].split);
     c->nact_split = t->nact_split;
     c->tiny_split = t->tiny_split;
     c->ens_chunks = t->ens_chunks > 0 ? t->ens_chunks : ens_chunks_default(c->prec);
