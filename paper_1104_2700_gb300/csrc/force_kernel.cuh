@@ -1644,7 +1644,13 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
     // and the launch as long as its dearest tile.  Near tiles are cut then;
     // the far loop's FP32 run of 64 is not: one unit does the whole tile, the
     // others nothing (which one rotates with the tile, since unit u of a tile
-    // is warp u of a CTA and a CTA's warps sit on different schedulers).  DS
+    // is warp u of a CTA and a CTA's warps sit on different schedulers).  Who
+    // does a tile must be the same answer in every warp that holds a unit of
+    // it, so the far test here leaves the guard out: a list may name a particle
+    // in two groups, and then some warps of the one already read the noise
+    // estimate that the other stores in this launch.  (The near limits come
+    // from a, j and the bound, which no force launch writes.)  With the guard
+    // on, the one unit takes the near path over the whole tile.  DS
     // and FP64, whose tiles are long (64 x ~250 dependent operations, ~15 us
     // for a warp alone): until each warp has UNITS units, so that the last
     // round of tiles is not mostly idle.
@@ -1863,15 +1869,22 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
         if constexpr (K::GUARDED) {
             // the far path when no lane's particle is in the tile, no lane
             // has the guard on and the tile is far from every lane's i
-            bool far = !mask_self && !guard_any;
+            bool far = !mask_self && (!guard_any || (CUTS && wl > 0));
             if (far) {
                 const float e2h = gi.e2.h;
 #pragma unroll
                 for (int q = 0; q < IT; ++q) far &= K::tile_far(buf, is[q], e2h);
                 far = __all_sync(0xffffffffu, far);
             }
+            const bool mine = !CUTS || !far || ((t ^ (t >> wl)) & ((1 << wl) - 1)) == 0;
+            if constexpr (CUTS) {
+                if (guard_any && far) {  // the near path over all of it or nothing
+                    u0 = 0, u1 = mine ? TJ / S : 0;
+                    far = false;
+                }
+            }
             if (far) {
-                if (!CUTS || ((t ^ (t >> wl)) & ((1 << wl) - 1)) == 0)
+                if (mine)
                     K::template far_tile<S>(buf, gi.e2, is, ac, sl);
             } else {
                 uint32_t nlo[IT], nhi[IT];

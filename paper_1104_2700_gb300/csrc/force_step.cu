@@ -275,6 +275,8 @@ __global__ void __launch_bounds__(ST_THREADS, K::MIN_CTAS) step_force_kernel(con
                 const bool mask_self =
                     __any_sync(0xffffffffu, is[0].p >= j0 && is[0].p < j0 + TJ);
                 const int u0 = wib * (TJ / ST_WARPS), u1 = u0 + TJ / ST_WARPS;
+                // (the same answer in every warp of the group: a block names no
+                // particle twice, so no other group stores its noise estimate)
                 bool far = !mask_self && !guard_any;
                 if (far) far = __all_sync(0xffffffffu, K::tile_far(buf, is[0], gi.e2.h));
                 if (far) {
