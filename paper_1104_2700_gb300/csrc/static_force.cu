@@ -87,9 +87,11 @@ __global__ void __launch_bounds__(4 * nb::TJ)
         rec[2][4 * slot + c] = vh;
         rec[3][4 * slot + c] = vl;
     } else {
-        const nb::Dsf gm = i < n ? nb::dsf_mass(G, m[i]) : nb::Dsf{0.f, 0.f};
-        rec[0][4 * slot + 3] = gm.hi;
-        rec[1][4 * slot + 3] = gm.lo;
+        // (in FP64: m alone may lie outside the range of a float)
+        const double gm = i < n ? G * m[i] : 0.0;
+        const float hi = __double2float_rn(gm);
+        rec[0][4 * slot + 3] = hi;
+        rec[1][4 * slot + 3] = __double2float_rn(gm - static_cast<double>(hi));
         rec[2][4 * slot + 3] = 0.f;
         rec[3][4 * slot + 3] = 0.f;
     }
