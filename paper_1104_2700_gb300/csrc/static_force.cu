@@ -60,11 +60,53 @@ Plan plan_for(int64_t n, int grid)
     return p;
 }
 
+__device__ __noinline__ void split_fp64(double x, uint32_t bound, float& hi, float& lo)
+{
+    nb::grid_split(x, nb::grid_quantum(bound), hi, lo);
+}
+
+// grid_split of x on the grid of `bound`, the same bits, on the FP32 and integer
+// pipes: |x| is cut exactly into its leading 24 bits and the other 29 (rest),
+// rounded to the grid from both, and the difference summed from exact parts.
+// Zeros are common (a cold start); a grid or an x whose parts leave FP32's
+// normal range takes the FP64 form.
+__device__ __forceinline__ void split(double x, uint32_t bound, float& hi, float& lo)
+{
+    const uint32_t hw = static_cast<uint32_t>(__double2hiint(x));
+    const uint32_t lw = static_cast<uint32_t>(__double2loint(x));
+    if (((hw & 0x7fffffffu) | lw) == 0u) {
+        hi = lo = 0.f;
+        return;
+    }
+    const uint32_t e = (hw >> 20) & 0x7ffu, eb = (bound >> 23) & 0xffu;
+    // |x| outside [2^-60, 2^61), or the grid's quantum outside [2^-121, 2^105]
+    if (e - (1023u - 60u) > 120u || eb - 27u > 226u) {
+        split_fp64(x, bound, hi, lo);
+        return;
+    }
+    float q, iq;
+    nb::grid_quantum_f(bound, q, iq);
+    const float xh =
+        __uint_as_float(((e - 1023u + 127u) << 23) | ((hw & 0xfffffu) << 3) | (lw >> 29));
+    const uint32_t rest = lw & 0x1fffffffu;
+    const float unit = __uint_as_float((e - 1075u + 127u) << 23);  // of rest
+    const float t = xh * iq;
+    float k = rintf(t);
+    if (t - k == 0.5f && rest) k += 1.f;  // not a tie
+    const float h = k * q;
+    float s, err;
+    nb::two_sum(__fsub_rn(xh, h), __uint2float_rn(rest >> 5) * (32.f * unit), s, err);
+    const float l = __fadd_rn(s, __fadd_rn(err, __uint2float_rn(rest & 31u) * unit));
+    hi = (hw >> 31) ? -h : h;
+    lo = (hw >> 31) ? -l : l;
+}
+
 // Predicted particles (device, n x 3 doubles) -> the double-single j layout
 // (grid-aligned splits on the grids of `bound`), with zero-mass ghosts far
 // away up to n_pad.  Four groups of 64 threads per tile, one per component and
-// one for the masses, on the FP32 pipes, as the predictor kernels; the FP64
-// splits of one thread per particle took 8.4 us at n = 8192.
+// one for the masses, as the predictor kernels, and the splits on the FP32
+// pipes: with FP64 splits the call took 82.8 us at n = 8192, 500 active, and
+// 86.9 with all of a particle in one thread.
 __global__ void __launch_bounds__(4 * nb::TJ)
     static_layout_kernel(int64_t n, const double* m, const double* r, const double* v, double G,
                          const uint32_t* bound, float4* L, int64_t n_pad)
@@ -75,12 +117,8 @@ __global__ void __launch_bounds__(4 * nb::TJ)
     if (c < 3) {
         float xh = static_cast<float>(nb::GHOST_POS), xl = 0.f, vh = 0.f, vl = 0.f;
         if (i < n) {
-            const double x = r[3 * i + c], u = v[3 * i + c];
-            float q, iq;
-            nb::grid_quantum_f(bound[0], q, iq);
-            nb::grid_split_ds(nb::dsf_of(x), q, iq, xh, xl);
-            nb::grid_quantum_f(bound[1], q, iq);
-            nb::grid_split_ds(nb::dsf_of(u), q, iq, vh, vl);
+            split(r[3 * i + c], bound[0], xh, xl);
+            split(v[3 * i + c], bound[1], vh, vl);
         }
         rec[0][4 * slot + c] = xh;
         rec[1][4 * slot + c] = xl;

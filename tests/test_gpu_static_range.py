@@ -42,3 +42,38 @@ def test_masses_that_only_g_brings_into_range(gpu, orc, G, scale):
     ref = orc.force(m, r, v, 4.0 / n, G=G, nthreads=os.cpu_count() or 1)
     for x, y in zip(got, ref):
         assert np.isfinite(x).all() and _err(x, y) < DS_BOUND
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-33, 0.0])
+def test_nearly_cold_start(gpu, orc, scale):
+    """Velocities whose grid quantum has no FP32 reciprocal (largest |v| below
+    2^-105 or so).  Their FP32 parts below 2^-126 flush to zero, so each velocity
+    is good to 2^-126 of itself and the jerk, against the largest, to a few
+    hundred such errors over the largest |v|."""
+    n = 1000
+    m, r, v = ics.plummer(n, 18)
+    v = v * (scale / np.abs(v).max())
+    acc, jerk, pot = _static(gpu, m, r, v, 4.0 / n, 1.0)
+    a0, j0, p0 = orc.force(m, r, v, 4.0 / n, nthreads=os.cpu_count() or 1)
+    assert _err(acc, a0) < DS_BOUND and _err(pot, p0) < DS_BOUND
+    assert np.isfinite(jerk).all()
+    if scale == 0.0:
+        assert not jerk.any()
+    else:
+        bound = max(DS_BOUND, 300 * 2.0 ** -126 / scale)
+        assert np.abs(jerk - j0).max() <= bound * np.abs(j0).max()
+
+
+@pytest.mark.parametrize("v_scale", [1.0, 1e25])
+def test_values_far_from_the_grid(gpu, orc, v_scale):
+    """Coordinates far below the grid's quantum beside ordinary ones, and
+    velocities above 2^60: the values that are not split on the FP32 pipes."""
+    n = 1000
+    m, r, v = ics.plummer(n, 19)
+    r[::7, 0], r[3::7, 1], r[5::7, 2] = 1e-25, -1e-30, 0.0
+    v[::5, 1], v[2::5, 2] = 1e-28, 0.0
+    v = v * v_scale
+    got = _static(gpu, m, r, v, 4.0 / n, 1.0)
+    ref = orc.force(m, r, v, 4.0 / n, nthreads=os.cpu_count() or 1)
+    for x, y in zip(got, ref):
+        assert _err(x, y) < DS_BOUND
