@@ -93,6 +93,7 @@ __device__ __forceinline__ void grid_quantum_f(uint32_t bound_bits, float& q, fl
         frexp(2.0 * static_cast<double>(__uint_as_float(bound_bits)), &e);
     else
         e = eb - 125;  // 2B = (1.f / 2) 2^(eb - 125), 1.f / 2 in [0.5, 1)
+    if (e < -100) e = -100;  // (both powers stay normal floats; such values travel in lo)
     q = ldexpf(1.f, e - 23);
     inv_q = ldexpf(1.f, 23 - e);
 }

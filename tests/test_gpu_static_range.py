@@ -1,6 +1,7 @@
-"""nb_force_static in units far from N-body units: its inputs are doubles, and
-only what the pair sums need (G m, the positions, the velocities) has to fit the
-FP32 pairs they are carried in.  Held to the DS bound, 1e-9 per particle."""
+"""nb_force_static, and NB_DS, in units far from N-body units: the inputs are
+doubles, and only what the pair sums need (G m, the positions, the velocities)
+has to fit the FP32 pairs they are carried in.  Held to the DS bound, 1e-9 per
+particle."""
 import ctypes
 import os
 
@@ -44,8 +45,9 @@ def test_masses_that_only_g_brings_into_range(gpu, orc, G, scale):
         assert np.isfinite(x).all() and _err(x, y) < DS_BOUND
 
 
+@pytest.mark.parametrize("call", ["static", "context"])
 @pytest.mark.parametrize("scale", [1e-30, 1e-33, 0.0])
-def test_nearly_cold_start(gpu, orc, scale):
+def test_nearly_cold_start(gpu, orc, scale, call):
     """Velocities whose grid quantum has no FP32 reciprocal (largest |v| below
     2^-105 or so).  Their FP32 parts below 2^-126 flush to zero, so each velocity
     is good to 2^-126 of itself and the jerk, against the largest, to a few
@@ -53,7 +55,14 @@ def test_nearly_cold_start(gpu, orc, scale):
     n = 1000
     m, r, v = ics.plummer(n, 18)
     v = v * (scale / np.abs(v).max())
-    acc, jerk, pot = _static(gpu, m, r, v, 4.0 / n, 1.0)
+    if call == "static":
+        acc, jerk, pot = _static(gpu, m, r, v, 4.0 / n, 1.0)
+    else:
+        with gpu.Context("ds") as c:
+            z = np.zeros((n, 3))
+            c.set_state(m, r, v, z, z, np.zeros(n), np.full(n, 2.0 ** -10), 4.0 / n, 0.02)
+            c.predict(0.0)
+            acc, jerk, pot = c.force(np.arange(n, dtype=np.int32))
     a0, j0, p0 = orc.force(m, r, v, 4.0 / n, nthreads=os.cpu_count() or 1)
     assert _err(acc, a0) < DS_BOUND and _err(pot, p0) < DS_BOUND
     assert np.isfinite(jerk).all()
