@@ -651,10 +651,12 @@ __global__ void __launch_bounds__(CLS_THREADS)
     }
     if (c == cl.k - 1 && tid == 0) {
         *sd.n_act = base.a + n;
-        if (gi > 0) {
-            cl.grp_tile0[base.b + g] = base.t + g * nt;
-            cl.plan_scalars[0] = base.b + g;
-            cl.plan_scalars[1] = base.t + g * nt;
+        if (gi > 0) {  // an empty plan if there were more groups than it holds
+            const int64_t G = base.b + g, T = base.t + g * nt;
+            const bool fits = G <= cl.max_groups;
+            if (fits) cl.grp_tile0[G] = T;
+            cl.plan_scalars[0] = fits ? G : 0;
+            cl.plan_scalars[1] = fits ? T : 0;
         }
     }
     if (n == 0) return;
