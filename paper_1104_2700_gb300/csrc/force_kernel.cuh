@@ -1675,6 +1675,14 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
             cR = gridDim.x / static_cast<uint32_t>(plan.G);  // G < gridDim.x / 4
             if (cR > rmax) cR = rmax;
             cta = plan.NT <= cR * FORCE_WARPS * CTA_MAX_TILES;
+            // The stream-K split cuts tiles too where UNITS > 1, and leaves no
+            // CTA out; from 33 groups on (no block of the default small variant,
+            // but any block of a launch that serves them all) it is the faster
+            // one unless the groups' equal shares fill the grid to 15 / 16
+            // (FP64, every particle active: N = 2944, 368 of 456 CTAs, 610
+            // against 520 us; N = 2700, 425 CTAs, 474 either way).
+            if (K::UNITS > 1 && plan.G > 32 && 16 * plan.G * cR < 15 * (int64_t)gridDim.x)
+                cta = false;
             if (!cta) wl = 0;
         }
         if (cta) {
