@@ -46,7 +46,7 @@ struct nb_ctx {
         int it = 1;
         int grid = 0;
         int split = 1;  // lanes per i (j split inside a warp)
-        bool full = true;  // as many CTAs per SM as fit
+        bool full = true;  // as many CTAs per SM as fit (set_full)
     } var[3];
     int32_t nact_split = 1024;
     int32_t tiny_split = 0;
@@ -682,6 +682,14 @@ std::vector<int32_t> internal_sorted(const nb_ctx* c, int32_t n_act, const int32
     return sorted;
 }
 
+// Whether the large variant takes as many CTAs per SM as fit: to be called
+// wherever it changes.
+void set_full(nb_ctx* c)
+{
+    nb_ctx::Variant& v = c->var[1];
+    v.full = v.grid / c->num_sms >= nb::force_ctas_per_sm(c->prec, v.it, v.split);
+}
+
 // Whether a kernel of the context may write doubles at p: null (not written),
 // or aligned device memory of the context's device.  Anything else goes through
 // a copy, which reports what it cannot reach.
@@ -935,8 +943,8 @@ nb_status nb_create(const nb_config* cfg, nb_ctx** out)
         c->var[v].it = it;
         c->var[v].split = split;
         c->var[v].grid = per_sm * c->num_sms;
-        c->var[v].full = per_sm >= occ;
     }
+    set_full(c);
     c->var[2] = c->var[0];  // no tiny variant until nb_autotune or nb_set_tuning sets one
     if (nb::force_setup(Prec::FP64, 1, 1) != cudaSuccess) return bail(NB_ECUDA);
     const int per_sm64 = nb::force_ctas_per_sm(Prec::FP64, 1, 1);
@@ -1437,12 +1445,13 @@ nb_status nb_set_ensemble(nb_ctx* c, int32_t k, const int64_t* offsets, const do
     nb_status s = ensure_capacity(c, n, n_pad, k);
     if (s != NB_OK) return s;
     // the ensemble plan cuts i-groups of one width for both variants, and
-    // there is no tiny one
+    // there is no tiny one; a large variant of another width would bring a grid
+    // chosen for its own occupancy, so it takes the small one's
     c->tiny_split = 0;
     c->var[2] = c->var[0];
     if (c->var[1].it != c->var[0].it || c->var[1].split != c->var[0].split) {
-        c->var[1].it = c->var[0].it;
-        c->var[1].split = c->var[0].split;
+        c->var[1] = c->var[0];
+        set_full(c);
         if ((s = ensure_force_scratch(c)) != NB_OK) return s;
     }
     c->eps = 0.0;  // per system: cl.eps2
@@ -1696,8 +1705,7 @@ nb_status nb_autotune(nb_ctx* c, nb_tuning* out)
     c->var[1] = {best[1]->it, best[1]->cps * c->num_sms, best[1]->split};
     c->var[2] = best[2] ? nb_ctx::Variant{best[2]->it, best[2]->cps * c->num_sms, best[2]->split}
                         : c->var[0];
-    c->var[1].full =
-        best[1]->cps >= nb::force_ctas_per_sm(c->prec, best[1]->it, best[1]->split);
+    set_full(c);
     c->nact_split = split_probe == 3 ? 1024 : 4096;
     c->tiny_split = tiny_probe == 0 ? 0 : tiny_probe == 1 ? 64 : 160;
     drop_graph(c);
@@ -1760,7 +1768,7 @@ nb_status nb_set_tuning(nb_ctx* c, const nb_tuning* t)
         const Shape& q = sh[v == 2 && t->tiny_split == 0 ? 0 : v];
         c->var[v] = {q.it, q.cps * c->num_sms, q.split};
     }
-    c->var[1].full = sh[1].cps >= nb::force_ctas_per_sm(c->prec, sh[1].it, sh[1].split);
+    set_full(c);
     c->nact_split = t->nact_split;
     c->tiny_split = t->tiny_split;
     c->ens_chunks = t->ens_chunks > 0 ? t->ens_chunks : ens_chunks_default(c->prec);
