@@ -1678,10 +1678,11 @@ __global__ void __launch_bounds__(FORCE_WARPS * 32, K::MIN_CTAS)
             // The stream-K split cuts tiles too where UNITS > 1, and leaves no
             // CTA out; from 33 groups on (no block of the default small variant,
             // but any block of a launch that serves them all) it is the faster
-            // one unless the groups' equal shares fill the grid to 15 / 16
-            // (FP64, every particle active: N = 2944, 368 of 456 CTAs, 610
-            // against 520 us; N = 2700, 425 CTAs, 474 either way).
-            if (K::UNITS > 1 && plan.G > 32 && 16 * plan.G * cR < 15 * (int64_t)gridDim.x)
+            // one unless the groups' equal shares fill 11 / 12 of the grid
+            // (every particle active, N = 2944, 368 of 456 CTAs: FP64 610
+            // against 515 us, DS 129 against 119; N = 3300, 416 CTAs: 682 / 627,
+            // 139 / 134; DS N = 1500, 423 CTAs: 62 / 66).
+            if (K::UNITS > 1 && plan.G > 32 && 12 * plan.G * cR < 11 * (int64_t)gridDim.x)
                 cta = false;
             if (!cta) wl = 0;
         }
