@@ -690,19 +690,68 @@ void set_full(nb_ctx* c)
     v.full = v.grid / c->num_sms >= nb::force_ctas_per_sm(c->prec, v.it, v.split);
 }
 
-// Whether a kernel of the context may write doubles at p: null (not written),
-// or aligned device memory of the context's device.  Anything else goes through
-// a copy, which reports what it cannot reach.
-bool on_this_device(const nb_ctx* c, const void* p)
+// The allocation that holds a device address (null: the driver does not say).
+using AddressRangeFn = int (*)(unsigned long long* base, size_t* size, unsigned long long p);
+AddressRangeFn address_range()
+{
+    static const AddressRangeFn fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault,
+                                             &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<AddressRangeFn>(f);
+    }();
+    return fn;
+}
+
+// Whether a kernel of the context may write k doubles at p: null (not written),
+// or aligned device memory of the context's device, all of it in the allocation
+// that p points into.  Anything else goes through a copy, which reports what it
+// cannot reach.
+bool on_this_device(const nb_ctx* c, const void* p, size_t k)
 {
     if (!p) return true;
-    if (reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0) return false;
+    const uintptr_t u = reinterpret_cast<uintptr_t>(p);
+    if (u % sizeof(double) != 0) return false;
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == c->device;
+    if (at.type != cudaMemoryTypeDevice || at.device != c->device) return false;
+    unsigned long long base = 0;
+    size_t size = 0;
+    return address_range() && address_range()(&base, &size, u) == 0 &&
+           u - base + k * sizeof(double) <= size;
+}
+
+// Whether nb_force's kernel may write its results to the caller's arrays itself:
+// they are this device's memory, and no two of them, nor one and the list, share
+// bytes (the copies come after the last read of the list, one array after the
+// other).
+bool direct_outputs(const nb_ctx* c, int32_t n_act, const int32_t* idx, const double* acc,
+                    const double* jerk, const double* pot)
+{
+    const size_t k = n_act;
+    if (!on_this_device(c, acc, 3 * k) || !on_this_device(c, jerk, 3 * k) ||
+        !on_this_device(c, pot, k))
+        return false;
+    const struct {
+        const void* p;
+        size_t bytes;
+    } a[4] = {{acc, 24 * k}, {jerk, 24 * k}, {pot, 8 * k}, {idx, 4 * k}};
+    for (int x = 0; x < 4; ++x)
+        for (int y = 0; y < x; ++y) {
+            if (!a[x].p || !a[y].p) continue;
+            const uintptr_t u = reinterpret_cast<uintptr_t>(a[x].p);
+            const uintptr_t v = reinterpret_cast<uintptr_t>(a[y].p);
+            if (u < v + a[y].bytes && v < u + a[x].bytes) return false;
+        }
+    return true;
 }
 
 nb_status validate_idx(nb_ctx* c, int32_t n_act, const int32_t* idx)
@@ -1213,10 +1262,9 @@ nb_status nb_force(nb_ctx* c, int32_t n_act, const int32_t* idx, double* acc, do
     } else if (n_act > 0) {
         // one launch: n_act as a parameter, and a device list in the caller's
         // numbering mapped to layout slots by the kernel itself, which also
-        // writes the caller's arrays where they are this device's memory
+        // writes the caller's arrays where it may
         Outputs out;
-        direct = on_device && on_this_device(c, acc) && on_this_device(c, jerk) &&
-                 on_this_device(c, pot);
+        direct = on_device && direct_outputs(c, n_act, idx, acc, jerk, pot);
         if (direct) out = {acc, jerk, pot};
         if ((s = run_force(c, c->prec, c->jl, on_device ? idx : c->idx_user, c->n_act_user,
                            n_act, on_device ? c->inv_dev : nullptr, out)) != NB_OK)
