@@ -365,10 +365,6 @@ nb_status check_status(nb_ctx* c)
     return fail(c, NB_ECUDA, "unknown device status 0x%x", st);
 }
 
-// Force on the active list idx[0..*n_act_dev).  In the context precision the
-// two launch variants go out back to back, each working only inside its
-// n_act window (the block size is read on the device); when the caller
-// knows n_act (n_act_host >= 0) only the matching variant is launched.
 nb::ForceArgs force_args(nb_ctx* c, Prec p, const nb::JLayout& jl, const int32_t* idx,
                          const int32_t* n_act_dev);
 
@@ -380,6 +376,11 @@ struct Outputs {
     double* pot = nullptr;
 };
 
+// Force on the active list idx[0..*n_act_dev).  When the caller knows n_act
+// (n_act_host >= 0) the variant whose window holds it is launched.  With the
+// block size on the device, one launch serves every size where the two variants
+// are one shape and its small-block build is good for all (ONE_BUILD_MAX_N);
+// else both go out, each working only inside its n_act window.
 nb_status run_force(nb_ctx* c, Prec p, const nb::JLayout& jl, const int32_t* idx,
                     const int32_t* n_act_dev, int32_t n_act_host = -1,
                     const int32_t* idx_map = nullptr, const Outputs& out = Outputs())

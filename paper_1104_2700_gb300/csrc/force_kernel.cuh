@@ -680,9 +680,8 @@ struct PolicyDS {
 // in space, and long runs of them raise the rounding of the run sums enough
 // to switch on the integration guard below for many more particles), near
 // pairs marked in a per-lane mask
-// during the FP32 pass and evaluated in double-single after it, each lane
-// walking its own list, so the warp runs the DS pair about
-// max-over-lanes(near pairs in the tile) times per tile.  Each run is folded
+// during the FP32 pass and evaluated in double-single after it, shared out over
+// the warp's lanes (near_pass).  Each run is folded
 // into double-single accumulators, so far-field rounding stays at the FP32
 // level of each term and never accumulates; the rsqrt estimate is refined
 // once through its residual.  Velocity differences of far pairs are taken
@@ -1019,7 +1018,13 @@ struct PolicyHybrid {
     // mask, or the warp shares out the list of all pairs (balanced).
     // Measured against every lane walking its own mask: a 32-particle block at
     // N = 16384 with its prediction 19.5 -> 16.6 us, every particle of
-    // N = 65536 8.33 -> 7.70 ms, block steps at N = 16384 57 -> 43 us each.
+    // N = 65536 8.33 -> 7.70 ms, block steps at N = 16384 57 -> 43 us each; the
+    // list (balanced) alone: 256 systems of 256-2048 particles, a force call on
+    // all of them, 2278 -> 1531 us.  It loses where nearly every lane's list is
+    // nearly full, thousands of systems of ~100 particles softened by half
+    // their size: 4500 of 64-128, 818 -> 995 us (855 with every lane walking
+    // its own mask in the older build); dearer estimates of its cost lost more
+    // elsewhere (1531 -> 1629 us).
     template <int S>
     __device__ static void near_pass(const unsigned char* buf, const Eps2& e2s,
                                      const I (&is)[IT], Acc (&ac)[IT], int lane,

@@ -252,11 +252,11 @@ cudaError_t predict_launch(const StateDev& st, Prec p, const JLayout& jl, double
                            const int32_t* n_act_dev, cudaStream_t s, const ClusterDev* cl)
 {
     if (st.n_pad <= 0) return cudaSuccess;
-    // Small blocks: the predictor is FP64-pipe bound per SM (GB300's FP64
-    // rate is a small fraction of FP32), so it should reach every SM.  One
-    // block is one tile of the j layout.
+    // One block is one tile of the j layout: the FP64 predictors are bound by
+    // the FP64 pipe of each SM (a small fraction of the FP32 rate), the
+    // double-single one by latency, so both should reach every SM.
     constexpr int threads = 64;
-    static_assert(threads == TJ, "the hybrid predictor reduces each tile in one block");
+    static_assert(threads == TJ, "a block per tile");
     const unsigned blocks = static_cast<unsigned>((st.n_pad + threads - 1) / threads);
     const int32_t* jsrc = cl ? cl->jsrc : nullptr;
     const int32_t* cof = cl ? cl->cluster_of : nullptr;

@@ -132,7 +132,9 @@ __device__ __forceinline__ void two_prod(float a, float b, float& p, float& e)
 // Grid-aligned double-single split.  Given a bound B on every |x| of one
 // layout, q = P 2^-23 with P the least power of two above 2B.  hi is x
 // rounded to a multiple of q (|hi| <= 2^23 q, so it fits a float exactly) and
-// lo = x - hi (|lo| <= q/2, kept to 24 bits: hi + lo is x to ~B 2^-47).  Since
+// lo = x - hi (|lo| <= q/2, kept to 24 bits: hi + lo is x to ~B 2^-47).  The
+// static call's layout is split so; the predictor's grid_split_ds rounds the
+// leading 24 bits of x only, so its |lo| can reach q.  Since
 // every hi part lies on the same grid and |hi_j - hi_i| <= 2^24 q, the FP32
 // difference of two hi parts is exact.  The factor 2 leaves room for values
 // that grow past B before the bound is raised; a value beyond 2B still splits
@@ -155,8 +157,9 @@ __device__ __forceinline__ void grid_split(double x, const GridQuantum& g, float
 }
 
 // (jh + jl) - (ih + il) for grid-aligned splits, as a normalised (dh, dl):
-// jh - ih is exact, and its magnitude is 0 or at least q >= |jl - il|, so
-// Fast2Sum renormalises exactly.
+// jh - ih is exact, and its magnitude is 0 or at least q.  |jl - il| is at most
+// q, or below 2q from grid_split_ds, so its exponent is no larger than that of
+// jh - ih, and Fast2Sum renormalises exactly.
 __device__ __forceinline__ void grid_diff(float jh, float jl, float ih, float il, float& dh,
                                           float& dl)
 {

@@ -53,7 +53,7 @@ struct StateDev {
     // [0] bound on every |position component|, [1] on every |velocity
     // component| (float bits, never decreasing): set from the whole state at
     // load, raised by the corrector.  They fix the grid of the j layout's
-    // double-single split (grid_split).
+    // double-single split (grid_split, grid_split_ds).
     uint32_t* bound = nullptr;
     // Hybrid precision: per particle, the far-field noise estimate of its
     // last force evaluation, negative when that evaluation was guarded
@@ -82,7 +82,7 @@ cudaError_t next_key_launch(const StateDev& st, cudaStream_t s);
 //   MIXED: arr[0] = float4 (x_hi, y_hi, z_hi, G m), arr[1] = float4 (x_lo,
 //          y_lo, z_lo, vx), arr[2] = float2 (vy, vz)
 //   Position (and DS velocity) hi/lo pairs are grid-aligned splits
-//   (grid_split): every hi part of the layout lies on one power-of-two grid.
+//   (grid_split_ds): every hi part of the layout lies on one power-of-two grid.
 //   DS:    arr[0] = float4 (x_hi, y_hi, z_hi, Gm_hi), arr[1] = float4
 //          (x_lo, y_lo, z_lo, Gm_lo), arr[2] = float4 (vx_hi, vy_hi, vz_hi,
 //          (Gm)^(2/3)), arr[3] = float4 (vx_lo, vy_lo, vz_lo, 0)

@@ -98,7 +98,9 @@ __device__ __forceinline__ void grid_quantum_f(uint32_t bound_bits, float& q, fl
     inv_q = ldexpf(1.f, 23 - e);
 }
 
-// x rounded to a multiple of q (hi) and the rest (lo); x.hi - hi is exact.
+// x rounded to a multiple of q (hi) and the rest (lo); x.hi - hi is exact.  The
+// rounding looks at x.hi alone, which lies within an ulp of x (at most q/2 while
+// |x| is within twice the bound), so |lo| < q, not q/2 as in grid_split.
 __device__ __forceinline__ void grid_split_ds(Dsf x, float q, float inv_q, float& hi, float& lo)
 {
     hi = rintf(x.hi * inv_q) * q;
