@@ -11,6 +11,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "nb_device.cuh"
 #include "nb_launch.h"
 #include "nbody.h"
@@ -691,20 +693,20 @@ void set_full(nb_ctx* c)
     v.full = v.grid / c->num_sms >= nb::force_ctas_per_sm(c->prec, v.it, v.split);
 }
 
-// The allocation that holds a device address (null: the driver does not say).
-using AddressRangeFn = int (*)(unsigned long long* base, size_t* size, unsigned long long p);
-AddressRangeFn address_range()
+// cuPointerGetAttributes (the runtime's call does not tell the allocation).
+using PointerAttributesFn = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+PointerAttributesFn pointer_attributes()
 {
-    static const AddressRangeFn fn = [] {
+    static const PointerAttributesFn fn = [] {
         void* f = nullptr;
         cudaDriverEntryPointQueryResult found;
-        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault,
-                                             &found) != cudaSuccess ||
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000,
+                                             cudaEnableDefault, &found) != cudaSuccess ||
             found != cudaDriverEntryPointSuccess) {
             cudaGetLastError();
             f = nullptr;
         }
-        return reinterpret_cast<AddressRangeFn>(f);
+        return reinterpret_cast<PointerAttributesFn>(f);
     }();
     return fn;
 }
@@ -717,16 +719,18 @@ bool on_this_device(const nb_ctx* c, const void* p, size_t k)
 {
     if (!p) return true;
     const uintptr_t u = reinterpret_cast<uintptr_t>(p);
-    if (u % sizeof(double) != 0) return false;
-    cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    if (at.type != cudaMemoryTypeDevice || at.device != c->device) return false;
+    if (u % sizeof(double) != 0 || !pointer_attributes()) return false;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned type = 0, managed = 1;
+    int device = -1;
     unsigned long long base = 0;
     size_t size = 0;
-    return address_range() && address_range()(&base, &size, u) == 0 &&
+    void* to[] = {&type, &managed, &device, &base, &size};
+    if (pointer_attributes()(5, what, to, u) != CUDA_SUCCESS) return false;
+    return type == CU_MEMORYTYPE_DEVICE && !managed && device == c->device && base <= u &&
            u - base + k * sizeof(double) <= size;
 }
 
