@@ -14,15 +14,16 @@ pytestmark = pytest.mark.gpu
 DS_BOUND = 1e-9
 
 
-def _static(gpu, m, r, v, eps, G):
+def _static(gpu, m, r, v, eps, G, n_act=None):
     torch = pytest.importorskip("torch")
     n = len(m)
+    k = n_act or n
     d = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (m, r, v)]
-    idx = torch.arange(n, dtype=torch.int32, device="cuda")
-    out = [torch.empty((n,) + s, dtype=torch.float64, device="cuda") for s in ((3,), (3,), ())]
+    idx = torch.arange(k, dtype=torch.int32, device="cuda")
+    out = [torch.empty((k,) + s, dtype=torch.float64, device="cuda") for s in ((3,), (3,), ())]
     torch.cuda.synchronize()
     p = [ctypes.c_void_p(t.data_ptr()) for t in d + [idx] + out]
-    assert gpu.nb_force_static(n, *p[:3], eps, G, n, *p[3:], None) == 0
+    assert gpu.nb_force_static(n, *p[:3], eps, G, k, *p[3:], None) == 0
     return [x.cpu().numpy() for x in out]
 
 
@@ -84,5 +85,17 @@ def test_values_far_from_the_grid(gpu, orc, v_scale):
     v = v * v_scale
     got = _static(gpu, m, r, v, 4.0 / n, 1.0)
     ref = orc.force(m, r, v, 4.0 / n, nthreads=os.cpu_count() or 1)
+    for x, y in zip(got, ref):
+        assert _err(x, y) < DS_BOUND
+
+
+@pytest.mark.parametrize("n_act", [1025, 1500, 1952, 2432])
+def test_blocks_above_a_thousand(gpu, orc, n_act):
+    """33 to 76 i-groups on this call's grid: equal shares of it or the even
+    split, by how the grid divides."""
+    n = 3000
+    m, r, v = ics.plummer(n, 22)
+    got = _static(gpu, m, r, v, 4.0 / n, 1.0, n_act)
+    ref = orc.force(m, r, v, 4.0 / n, idx=np.arange(n_act), nthreads=os.cpu_count() or 1)
     for x, y in zip(got, ref):
         assert _err(x, y) < DS_BOUND
