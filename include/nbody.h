@@ -136,23 +136,24 @@ void nb_config_init(nb_config* cfg);
  * returns at once: as two parallel branches where the large shape takes all
  * the CTAs that fit, one after the other where it does not.  Where the two
  * shapes are the same, with one i per thread, it is one launch (except
- * NB_HYBRID and NB_HYBRID_SPJ on one system above 8192 particles), and in
- * those precisions one system of at most 1536 particles, with one i per
- * thread and no j split in both shapes, takes select, prediction and force in
- * one launch on the small shape's CTAs, for blocks of every size.  The tiny
- * shape is never a block step's, since a third branch costs it more than the
- * shape saves.  i_per_thread is the i-tile per lane; j_split the lanes that
- * share one i, each taking every j_split-th j of a tile (an i-group is 32
- * i_per_thread / j_split particles); ctas_per_sm sets the persistent grid,
- * which fixes how far each i-group's j range is split across warps.  An
- * ensemble context uses one i-tile and one j split for both shapes (its force
- * plan is cut once per block) and no tiny shape.  An ensemble's force launch
- * cuts its (i-group, j tile) pairs into ens_chunks chunks per warp: with 1
- * each warp takes one contiguous range; with more (by default 4 for the
- * hybrid precisions, whose tiles differ several-fold in cost), each warp's
- * first chunk is its own and the rest go to warps in the order they come
- * free.  The *_us fields give the force time the autotuner measured for the
- * chosen shapes on their probe blocks (tiny_us 0 without a tiny shape). */
+ * NB_HYBRID and NB_HYBRID_SPJ on one system above 8192 particles, or with one
+ * CTA per SM), and in those precisions one system of at most 1536 particles,
+ * with one i per thread and no j split in both shapes, takes select,
+ * prediction and force in one launch on the small shape's CTAs, for blocks of
+ * every size.  The tiny shape is never a block step's, since a third branch
+ * costs it more than the shape saves.  i_per_thread is the i-tile per lane;
+ * j_split the lanes that share one i, each taking every j_split-th j of a
+ * tile (an i-group is 32 * i_per_thread / j_split particles); ctas_per_sm sets
+ * the persistent grid, which fixes how far each i-group's j range is split
+ * across warps.  An ensemble context uses one i-tile and one j split for both
+ * shapes (its force plan is cut once per block) and no tiny shape.  An
+ * ensemble's force launch cuts its (i-group, j tile) pairs into ens_chunks
+ * chunks per warp: with 1 each warp takes one contiguous range; with more (by
+ * default 4 for the hybrid precisions, whose tiles differ several-fold in
+ * cost), each warp's first chunk is its own and the rest go to warps in the
+ * order they come free.  The *_us fields give the force time the autotuner
+ * measured for the chosen shapes on their probe blocks (tiny_us 0 without a
+ * tiny shape). */
 typedef struct nb_tuning {
     int32_t small_i_per_thread;
     int32_t small_ctas_per_sm;

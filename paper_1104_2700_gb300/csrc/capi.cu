@@ -128,7 +128,11 @@ constexpr int GRAPH_STEPS = 32;  // block steps per replay of the step graph
 // two branches with a fork and a join (~1.5 us of a ~30 us block step).  For DS
 // and FP64 that build runs large blocks at the plain build's speed (N = 16384,
 // every particle, DS: 2.12 against 2.11 ms); for HYBRID it is slower there (957
-// against 816 us), so only systems whose blocks are small take it.
+// against 816 us), so only systems whose blocks are small take it, and none on a
+// grid of one CTA per SM, where that build's large blocks have no other CTA to
+// hide behind (N = 6000, every particle, eps = 1/2: 429 us a block step, 335 in
+// two branches; blocks of a few tens 50.5 and 53.2; on two CTAs per SM 260 / 211
+// and 50.1 / 52.8).
 constexpr int64_t ONE_BUILD_MAX_N = 8192;
 
 void drop_graph(nb_ctx* c)
@@ -419,8 +423,10 @@ nb_status run_force(nb_ctx* c, Prec p, const nb::JLayout& jl, const int32_t* idx
         return NB_OK;
     }
     const nb_ctx::Variant &v0 = c->var[0], &v1 = c->var[1];
+    const bool one_build = !nb::is_hybrid(c->prec) ||
+                           (c->n <= ONE_BUILD_MAX_N && v0.grid >= 2 * c->num_sms);
     if (v0.it == v1.it && v0.split == v1.split && v0.grid == v1.grid &&
-        (c->ens || (v0.it == 1 && (!nb::is_hybrid(c->prec) || c->n <= ONE_BUILD_MAX_N)))) {
+        (c->ens || (v0.it == 1 && one_build))) {
         f.it = v0.it;
         f.split = v0.split;
         f.grid = v0.grid;

@@ -1,4 +1,7 @@
-"""The force launches of an ensemble's block step, counted in a captured graph.
+"""The force launches of a block step, counted in a captured graph.
+
+HYBRID on a grid of one CTA per SM keeps its two builds apart; with more, up to 8192
+particles, the small-block build serves every block in one launch.
 
 An ensemble has one i-tile for blocks of every size.  A MIXED context's default
 large variant has another (two i per lane), so nb_set_ensemble replaces it, and
@@ -41,5 +44,18 @@ def test_mixed_variants_become_one(gpu):
         assert _nodes(torch, stream, lambda: c.block_step(1.0)) == 5
         c.set_particles(m1, r1, v1, 0.01, 0.02)
         assert _nodes(torch, stream, lambda: c.block_step(1.0)) == 4
+        c.block_step(1.0)
+        c.synchronize()
+
+
+@pytest.mark.parametrize("ctas,nodes", [(0, 4), (2, 4), (1, 5)])
+def test_hybrid_builds(gpu, ctas, nodes):
+    torch = pytest.importorskip("torch")
+    m, r, v = ics.plummer(3000, 2)
+    stream = torch.cuda.Stream()
+    with gpu.Context("hybrid", stream=stream, ctas_per_sm=ctas) as c:
+        c.set_particles(m, r, v, 0.01, 0.02)
+        # select, prediction, one force launch or two, corrector
+        assert _nodes(torch, stream, lambda: c.block_step(1.0)) == nodes
         c.block_step(1.0)
         c.synchronize()
